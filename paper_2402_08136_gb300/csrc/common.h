@@ -103,6 +103,12 @@ struct Op {
     // dev_off_tcw: the widened form's blob (complex64 device data)
     std::vector<int> tc_pads;
     size_t dev_off_tcw = 0;
+    // complex128 dense op that runs as exact digit products on the tensor cores (dense_f64.cu; its
+    // digits at dev_off_tc[1]): entries of U are below 2^f64_su, bit r of f64_keep: row r is row r
+    // of the identity
+    bool has_f64 = false;
+    int f64_su = 0;
+    unsigned long long f64_keep = 0;
     bool real_u = false;        // OP_DENSE: every entry of U is real (SIMT kernels use 2 FMAs per entry)
 };
 
@@ -191,6 +197,12 @@ void dense_tc_pack_real7(const std::vector<cd> &U, unsigned char *out);
 bool launch_dense_tc_real7(void *state, int n, const std::vector<int> &targets, const std::vector<int> &controls,
                            const void *Bdev, int sms, cudaStream_t st, double *sums = nullptr, int hi_bit = 0,
                            bool *sums_written = nullptr);
+// dense_f64.cu: complex128 dense gates as exact digit products on the tensor cores
+bool dense_f64_applies(const Op &op);
+size_t dense_f64_blob_bytes(const Op &op);
+void dense_f64_pack(Op &op, unsigned char *out);  // sets op.f64_su, op.f64_keep
+// Ut: U in FP64, transposed; false (nothing launched) when the state has too few groups
+bool launch_dense_f64(void *state, int n, const Op &op, const void *dig, const void *Ut, int sms, cudaStream_t st);
 // batched.cu: plan (host image) / instantiate (device tables) / launch / results, for the pool
 struct BatchImage;
 bool batch_supported(const qsim_circuit *c);  // every op runs in the batched executor

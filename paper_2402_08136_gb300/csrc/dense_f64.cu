@@ -1,0 +1,593 @@
+// Dense k-qubit gates on a complex128 state (sm_103a) as exact fixed-point products on the
+// tensor cores.
+//
+// What bounds the plain form: FP64 runs at 2 fused multiply-adds per clock and SM on this GPU, so
+// the 4 2^k of them that a complex128 amplitude needs take 2 2^k clocks per SM, against 1.5 clocks
+// for its 32 bytes of HBM traffic: every width from k = 1 up is bound by the FP64 pipe, by a factor
+// of 80 at k = 6.  The split used here (Ozaki, Ogita, Oishi & Rump, "Error-free transformations of
+// matrix multiplication by using fast routines of matrix multiplication and its applications",
+// Numerical Algorithms 2012) moves the products to the tensor cores without giving up precision:
+//   - the reals of a group (the 2^k amplitudes that differ in the target bits) are written as
+//     62-bit integers relative to the group's largest exponent, and those as eight signed base-256
+//     digits; U's entries likewise, relative to its largest entry (on the host, once);
+//   - a digit is exact in FP16, a product of two has 15 bits, and the FP32 accumulator of the MMA
+//     adds up to 2^10 of them exactly (all sums stay integers of at most 2^24): the 36 digit pairs
+//     (i, j) with i + j <= 7 go to the eight accumulators i + j;
+//   - the eight sums are put together in 64-bit integer arithmetic and rounded once to FP64.
+// What is left out (pairs with i + j > 7, bits below 2^-62 of the group's largest value) is below
+// 2^-57 of the largest product; the plain form rounds after every one of its 2 2^k additions.
+// All of it is integer and tensor work; the FP64 pipe only does the final conversion.
+//
+// A warp owns 8 groups (the N columns of m16n8k16; 4 groups x {re, im} for a real U).  The MMA's B
+// fragment wants, per lane, a pair of rows of one column, and which amplitude is which row is free,
+// so every lane loads its amplitudes straight from HBM into the fragment's place: there is no
+// shared-memory stage, no barrier and no exchange but the quad's maximum.  The accumulator's rows
+// are output amplitudes, written back in place.  U's digits sit in shared memory in fragment order.
+// Group bits are the lowest free qubits, so a warp's load covers whole 128-byte lines.
+//
+// Not all gates take this form (dense_f64_applies): one whose rows are mostly zeros keeps the plain
+// kernel, which is exact on permutations; rows that are rows of the identity are not written at all.
+// A tile with a group that is not finite, or whose largest exponent is far from 1, is computed in
+// the plain FP64 form by the same warp (plain_tile).
+#include <cuda_runtime.h>
+#include <cuda_fp16.h>
+
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+
+#include "common.h"
+
+namespace qsim {
+namespace f64 {
+
+constexpr int kMaxFix = 40;
+constexpr int kDigits = 8;
+constexpr int kMinExp = 200, kMaxExp = 1900;  // biased exponents of a group's largest value that take the split
+
+struct Args {
+    void *psi;
+    const uint4 *dig;            // U's digits in fragment order (pack_digits)
+    const double2 *Ut;           // U transposed, FP64 (plain_tile)
+    long long ntasks;
+    unsigned long long cmask;
+    unsigned long long keep;     // bit r set: row r of U is row r of the identity (not written)
+    int su;                      // U = (integers) 2^(su - 62)
+    int k;                       // the gate's own targets (below 3: the rest of the 8 amplitudes are group bits)
+    int real_u;
+    int nfix;
+    int fix[kMaxFix];            // ascending: targets, controls, group bits inside a task
+    long long amp[128];          // byte offset of amplitude a of a group
+    long long col[8];            // byte offset of group column 0..7 (0..3 for a real U)
+    long long tile[4];           // byte offset of the task's tiles
+};
+
+template <int K, bool REALU, int TBITS = -1>
+struct Cfg {
+    static constexpr int D = 1 << K;                   // amplitudes per group
+    static constexpr bool RF = K == 3 && !REALU;       // real form: one m-tile of (re, im) rows
+    static constexpr int MT = RF ? 1 : D / 16;         // m-tiles
+    static constexpr int KS = RF ? 1 : D / 16;         // k-steps
+    static constexpr int TABS = RF || REALU ? 1 : 3;   // U | Re U, Im U, -Im U
+    static constexpr int TAB = MT * KS * kDigits * 32; // uint4 per table
+    static constexpr int GB = REALU ? 2 : 3;           // group bits of a tile
+    static constexpr int RED = REALU ? D : 2 * D;      // terms of a sum
+    static constexpr bool BIAS = RED <= 32;            // sums below 2^22: read back without a conversion
+    static constexpr int SH = RED > 64 ? 13 : 12;      // bits dropped from the 2^-68 sum
+    // tiles per task: up to 8 amplitudes (16 reals) per lane in flight; states with too few tasks for
+    // the warps of the chip take one tile per task
+    static constexpr int TBMAX = REALU ? (K == 4 ? 2 : K == 5 ? 1 : 0) : (K == 3 ? 2 : K == 4 ? 1 : 0);
+    static constexpr int TB = TBITS < 0 ? TBMAX : TBITS;
+    static constexpr int NT = 1 << TB;
+    static constexpr int EPL = REALU ? D / 4 : D / 2;  // reals per lane and tile
+    static constexpr bool PREFETCH = EPL * NT <= 16;
+    static constexpr int THREADS = K == 6 && !REALU ? 256 : (K >= 5 ? 384 : 512);
+    static constexpr int SMEM = TABS * TAB * 16;
+};
+
+__device__ __forceinline__ void mma(float (&d)[4], const uint4 &a, unsigned b0, unsigned b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
+}
+
+__device__ __forceinline__ unsigned mag_bits(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
+
+// x as a 62-bit integer relative to 2^(E + 1) (E: a biased exponent not below x's), plus 128 in
+// every byte: byte i is digit i + 128 of the signed base-256 form, -128 <= digit <= 127
+__device__ __forceinline__ unsigned long long fixed_bytes(double x, int E) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const int s = E - (int)((hi >> 20) & 0x7ffu);
+    const unsigned mh = (__funnelshift_l(lo, hi, 9) & 0x1fffffffu) | 0x20000000u;
+    unsigned long long v = ((unsigned long long)mh << 32) | (lo << 9);
+    asm("shr.u64 %0, %0, %1;" : "+l"(v) : "r"(s));  // 0 from 64 on
+    const long long sg = (long long)((int)hi >> 31);
+    return (v ^ (unsigned long long)sg) + (0x8080808080808080ull - (unsigned long long)sg);
+}
+
+// The digits of two reals as FP16 pairs: out[i] = (digit i of a, digit i of b), i = 0 the highest.
+// A byte under 0x64 is FP16 1024 + byte.
+__device__ __forceinline__ void digit_pairs(unsigned long long a, unsigned long long b, unsigned (&out)[kDigits]) {
+    const __half2 off = __floats2half2_rn(1152.f, 1152.f);
+#pragma unroll
+    for (int w = 0; w < 2; w++) {
+        const unsigned x = w ? (unsigned)a : (unsigned)(a >> 32), y = w ? (unsigned)b : (unsigned)(b >> 32);
+        const unsigned t[2] = {__byte_perm(x, y, 0x7362), __byte_perm(x, y, 0x5140)};  // bytes 2, 3 and 0, 1
+#pragma unroll
+        for (int i = 0; i < 4; i++) {  // digit 4 w + i is byte 3 - i of the word
+            const unsigned h = __byte_perm(t[i >> 1], 0x64646464u, (i & 1) ? 0x4140 : 0x4342);
+            const __half2 r = __hsub2(*reinterpret_cast<const __half2 *>(&h), off);
+            out[4 * w + i] = *reinterpret_cast<const unsigned *>(&r);
+        }
+    }
+}
+
+constexpr float kBiasF = 12582912.0f;  // 1.5 2^23: an FP32 sum started there has its integer in its low bits
+
+// sum_t acc[t] 2^(8 (7 - t)) / 2^SH, rounded to FP64, times 2^(ex - 1023) (0 for a zero sum)
+template <typename C>
+__device__ __forceinline__ double join(const float (&acc)[kDigits], int ex) {
+    long long T;
+    if constexpr (C::BIAS) {
+        int h[4];
+#pragma unroll
+        for (int p = 0; p < 4; p++)
+            h[p] = (int)((__float_as_uint(acc[2 * p]) << 8) + __float_as_uint(acc[2 * p + 1]) - 257u * 0x4B400000u +
+                         (p == 3 ? 1u << (C::SH - 1) : 0u));
+        T = (long long)h[2] * (1 << (16 - C::SH)) + (long long)(h[3] >> C::SH);
+        T += (long long)h[1] * (1 << (32 - C::SH));
+        T += (long long)((unsigned long long)(unsigned)(h[0] << (16 - C::SH)) << 32);
+    } else {
+        long long p[2];
+#pragma unroll
+        for (int w = 0; w < 2; w++) {
+            p[w] = (long long)__float2int_rn(acc[4 * w]) * (1 << 24) + (long long)__float2int_rn(acc[4 * w + 1]) * (1 << 16);
+            p[w] += (long long)__float2int_rn(acc[4 * w + 2]) * (1 << 8) + (long long)__float2int_rn(acc[4 * w + 3]);
+        }
+        T = (p[0] << (32 - C::SH)) + ((p[1] + (1 << (C::SH - 1))) >> C::SH);
+    }
+    const double d = (double)T;
+    const int hi = __double2hiint(d);
+    return __hiloint2double(hi ? hi + (ex << 20) : 0, __double2loint(d));
+}
+
+// One tile in the plain FP64 form, U's columns in order as the plain kernels add them.
+template <int K, bool REALU>
+__device__ __noinline__ void plain_tile(const Args &a, char *base, int lane) {
+    constexpr int D = 1 << K, GB = Cfg<K, REALU>::GB;
+    constexpr int LPG = 32 >> GB, OUT = D / LPG;  // lanes per group, outputs per lane
+    char *p = base + a.col[lane / LPG];
+    const int D0 = 1 << a.k;  // bits from a.k on are group bits
+    double2 y[OUT];
+#pragma unroll 1
+    for (int o = 0; o < OUT; o++) {
+        const int row = lane % LPG + o * LPG, r = row & (D0 - 1);
+        double2 s = make_double2(0.0, 0.0);
+#pragma unroll 1
+        for (int c = 0; c < D0; c++) {
+            const double2 x = *reinterpret_cast<const double2 *>(p + a.amp[(row & ~(D0 - 1)) | c]);
+            const double2 u = a.Ut[c * D0 + r];
+            s.x = fma(u.x, x.x, s.x);
+            if (!a.real_u) s.x = fma(-u.y, x.y, s.x);
+            s.y = fma(u.x, x.y, s.y);
+            if (!a.real_u) s.y = fma(u.y, x.x, s.y);
+        }
+        y[o] = s;
+    }
+    __syncwarp();  // every output of the tile is computed before any is stored
+#pragma unroll 1
+    for (int o = 0; o < OUT; o++) {
+        *reinterpret_cast<double2 *>(p + a.amp[lane % LPG + o * LPG]) = y[o];
+    }
+    __syncwarp();
+}
+
+template <int K, bool REALU, int TBITS>
+__global__ void __launch_bounds__(Cfg<K, REALU>::THREADS, 1) dense_f64_kernel(const __grid_constant__ Args a) {
+    using C = Cfg<K, REALU, TBITS>;
+    constexpr int NT = C::NT, EPL = C::EPL, KS = C::KS;
+    extern __shared__ __align__(16) uint4 tabs[];  // [TABS][MT][KS][digit][lane]
+    const int tid = threadIdx.x, lane = tid & 31, q = lane & 3, n = lane >> 2;
+    for (int i = tid; i < C::TAB * (C::TABS == 3 ? 2 : 1); i += C::THREADS) {
+        uint4 v = a.dig[i];
+        tabs[i] = v;
+        if (C::TABS == 3 && i >= C::TAB) {  // -Im U
+            v.x ^= 0x80008000u;
+            v.y ^= 0x80008000u;
+            v.z ^= 0x80008000u;
+            v.w ^= 0x80008000u;
+            tabs[i + C::TAB] = v;
+        }
+    }
+    __syncthreads();
+    const long long warps = (long long)gridDim.x * (C::THREADS / 32);
+    // B column n: group (n mod 2) 4 + n / 2 (the store of one accumulator column then covers the
+    // lowest group bits), or re / im of group n / 2 for a real U
+    const long long in_off = REALU ? a.col[n >> 1] + 8 * (n & 1) : a.col[(n & 1) * 4 + (n >> 1)];
+    const long long in_lane = in_off + a.amp[q], out_lane = a.amp[n] + a.col[q];
+    char *psi = static_cast<char *>(a.psi);
+
+    double x[NT][EPL];  // this lane's reals: EPL / 2 amplitudes of one group, or EPL parts for a real U
+    auto task_base = [&](long long t) -> char * {
+        unsigned long long g = (unsigned long long)t;
+        for (int i = 0; i < a.nfix; i++) {
+            const int p = a.fix[i];
+            g = ((g >> p) << (p + 1)) | (g & ((1ull << p) - 1ull));
+        }
+        return psi + 16 * (g | a.cmask);
+    };
+    auto load = [&](long long t, double(&v)[NT][EPL]) {
+        const char *p = task_base(t) + in_lane;
+#pragma unroll
+        for (int i = 0; i < NT; i++)
+            if constexpr (REALU) {
+#pragma unroll
+                for (int e = 0; e < EPL; e++) v[i][e] = __ldcs(reinterpret_cast<const double *>(p + a.tile[i] + a.amp[4 * e]));
+            } else {
+#pragma unroll
+                for (int e = 0; e < EPL / 2; e++) {
+                    const double2 z = __ldcs(reinterpret_cast<const double2 *>(p + a.tile[i] + a.amp[4 * e]));
+                    v[i][2 * e] = z.x;
+                    v[i][2 * e + 1] = z.y;
+                }
+            }
+    };
+    long long t = (long long)blockIdx.x * (C::THREADS / 32) + (tid >> 5);
+    if (C::PREFETCH && t < a.ntasks) load(t, x);
+    for (; t < a.ntasks; t += warps) {
+        if (!C::PREFETCH) load(t, x);
+        char *base = task_base(t);
+#pragma unroll
+        for (int i = 0; i < NT; i++) {
+            char *tb = base + a.tile[i], *ob = tb + out_lane;
+            // exponent of each column's largest value: over the quad, or for narrow gates (RF, k < 3)
+            // over the amplitudes that share the bits from k on
+            unsigned m0 = 0, m1 = 0;
+            if constexpr (C::RF) {
+                m0 = max(mag_bits(x[i][0]), mag_bits(x[i][1]));
+                m1 = max(mag_bits(x[i][2]), mag_bits(x[i][3]));
+                m0 = max(m0, __shfl_xor_sync(~0u, m0, 1));
+                m1 = max(m1, __shfl_xor_sync(~0u, m1, 1));
+                if (a.k >= 2) {
+                    m0 = max(m0, __shfl_xor_sync(~0u, m0, 2));
+                    m1 = max(m1, __shfl_xor_sync(~0u, m1, 2));
+                }
+                if (a.k >= 3) m0 = m1 = max(m0, m1);
+            } else {
+#pragma unroll
+                for (int e = 0; e < EPL; e++) m0 = max(m0, mag_bits(x[i][e]));
+                m0 = max(m0, __shfl_xor_sync(~0u, m0, 1));
+                m0 = max(m0, __shfl_xor_sync(~0u, m0, 2));
+                m1 = m0;
+            }
+            const int E0 = m0 ? (int)(m0 >> 20) : 1023, E1 = m1 ? (int)(m1 >> 20) : 1023;
+            bool fits = E0 >= kMinExp && E0 <= kMaxExp && E1 >= kMinExp && E1 <= kMaxExp;
+            if (m0 == 0 || m1 == 0) {  // all zero, or denormals whose high words are 0
+                unsigned low = 0;
+#pragma unroll
+                for (int e = 0; e < EPL; e++) low |= (unsigned)__double2loint(x[i][e]) & (mag_bits(x[i][e]) ? 0u : ~0u);
+                fits = fits && low == 0;
+            }
+            unsigned br[KS][2][kDigits], bi[REALU || C::RF ? 1 : KS][2][kDigits];
+            if constexpr (C::RF) {
+                digit_pairs(fixed_bytes(x[i][0], E0), fixed_bytes(x[i][1], E0), br[0][0]);
+                digit_pairs(fixed_bytes(x[i][2], E1), fixed_bytes(x[i][3], E1), br[0][1]);
+            } else {
+#pragma unroll
+                for (int s = 0; s < KS; s++)
+#pragma unroll
+                    for (int h = 0; h < 2; h++) {
+                        const int e = 4 * s + 2 * h;  // this lane's entries e, e + 1 of the k-step
+                        if constexpr (REALU) {
+                            digit_pairs(fixed_bytes(x[i][e], E0), fixed_bytes(x[i][e + 1], E0), br[s][h]);
+                        } else {
+                            digit_pairs(fixed_bytes(x[i][2 * e], E0), fixed_bytes(x[i][2 * e + 2], E0), br[s][h]);
+                            digit_pairs(fixed_bytes(x[i][2 * e + 1], E0), fixed_bytes(x[i][2 * e + 3], E0), bi[s][h]);
+                        }
+                    }
+            }
+            if (C::PREFETCH && i == NT - 1 && t + warps < a.ntasks) load(t + warps, x);
+            if (!__all_sync(~0u, fits)) {
+                plain_tile<K, REALU>(a, tb, lane);
+                continue;
+            }
+            // result exponents of this lane's two accumulator columns 2 q, 2 q + 1 (and row n)
+            const int ep = E0 | (E1 << 16);
+            const int src = 8 * q + (C::RF && a.k < 2 ? (n & 2) : 0);
+            int ex[2];
+#pragma unroll
+            for (int j = 0; j < 2; j++) {
+                const int v = __shfl_sync(~0u, ep, src + 4 * j);
+                ex[j] = (C::RF && n >= 4 ? v >> 16 : v & 0xffff) - 1022 + a.su - (68 - C::SH);
+            }
+            float acc[4][kDigits];
+            auto clear = [&] {
+#pragma unroll
+                for (int c = 0; c < 4; c++)
+#pragma unroll
+                    for (int d = 0; d < kDigits; d++) acc[c][d] = C::BIAS ? kBiasF : 0.f;
+            };
+            auto step = [&](const uint4 *tab, const unsigned(&b)[2][kDigits]) {
+#pragma unroll
+                for (int j = 0; j < kDigits; j++) {
+                    const uint4 u = tab[j * 32 + lane];
+#pragma unroll
+                    for (int d = 0; d + j < kDigits; d++) {
+                        float v[4] = {acc[0][d + j], acc[1][d + j], acc[2][d + j], acc[3][d + j]};
+                        mma(v, u, b[0][d], b[1][d]);
+#pragma unroll
+                        for (int c = 0; c < 4; c++) acc[c][d + j] = v[c];
+                    }
+                }
+            };
+            if constexpr (C::RF) {
+                clear();
+                step(tabs, br[0]);
+#pragma unroll
+                for (int j = 0; j < 2; j++) {  // amplitude n of group q + 4 j
+                    const double2 y = make_double2(join<C>(acc[j], ex[j]), join<C>(acc[2 + j], ex[j]));
+                    if (!((a.keep >> n) & 1ull))
+                        __stcs(reinterpret_cast<double2 *>(ob + a.col[4 * j]), y);
+                }
+            } else {
+#pragma unroll 1
+                for (int mt = 0; mt < C::MT; mt++) {
+                    const uint4 *tu = tabs + mt * KS * kDigits * 32;
+                    if constexpr (REALU) {
+                        clear();
+#pragma unroll
+                        for (int s = 0; s < KS; s++) step(tu + s * kDigits * 32, br[s]);
+#pragma unroll
+                        for (int h = 0; h < 2; h++) {  // amplitudes n and n + 8 of group q
+                            const int row = 16 * mt + 8 * h + n;
+                            const double2 y = make_double2(join<C>(acc[2 * h], ex[0]), join<C>(acc[2 * h + 1], ex[1]));
+                            if (!((a.keep >> row) & 1ull))
+                                __stcs(reinterpret_cast<double2 *>(ob + a.amp[16 * mt + 8 * h]), y);
+                        }
+                    } else {
+                        double re[4];
+                        clear();
+#pragma unroll
+                        for (int s = 0; s < KS; s++) {
+                            step(tu + s * kDigits * 32, br[s]);
+                            step(tu + 2 * C::TAB + s * kDigits * 32, bi[s]);
+                        }
+#pragma unroll
+                        for (int c = 0; c < 4; c++) re[c] = join<C>(acc[c], ex[c & 1]);
+                        clear();
+#pragma unroll
+                        for (int s = 0; s < KS; s++) {
+                            step(tu + C::TAB + s * kDigits * 32, br[s]);
+                            step(tu + s * kDigits * 32, bi[s]);
+                        }
+#pragma unroll
+                        for (int c = 0; c < 4; c++) {  // amplitudes n and n + 8 of groups q and q + 4
+                            const int row = 16 * mt + 8 * (c >> 1) + n;
+                            const double2 y = make_double2(re[c], join<C>(acc[c], ex[c & 1]));
+                            if (!((a.keep >> row) & 1ull))
+                                __stcs(reinterpret_cast<double2 *>(ob + a.col[4 * (c & 1)] + a.amp[16 * mt + 8 * (c >> 1)]), y);
+                        }
+                    }
+                }
+            }
+        }
+    }
+}
+
+// u / 2^(su - 62) as signed base-256 digits, -127 <= digit <= 128 (so that no product of a digit
+// with one of the state's reaches +2^14), highest first, as FP16 bit patterns
+static void digits_of(double u, double scale, unsigned short (&d)[kDigits]) {
+    struct Half {
+        unsigned short bits[256];
+        Half() {
+            for (int v = 0; v < 256; v++) {
+                const __half h = __float2half_rn((float)(v - 127));
+                std::memcpy(&bits[v], &h, 2);
+            }
+        }
+    };
+    static const Half half;
+    long long w = std::llrint(u * scale);  // at most 2^62
+    for (int i = kDigits - 1; i >= 0; i--) {
+        const int b = (int)((w + 127) & 255);
+        d[i] = half.bits[b];
+        w = (w + 127 - b) / 256;
+    }
+}
+
+// kernel width of a gate: at least 3 targets, 4 for a real U
+static int width_of(const Op &op) {
+    const int k = (int)op.targets.size();
+    return k <= 3 ? 3 : k;
+}
+static bool real_form(const Op &op) { return op.real_u && op.targets.size() >= 4; }
+
+template <int K, bool REALU>
+static void pack_digits(const Op &op, int su, unsigned char *out) {
+    using C = Cfg<K, REALU>;
+    const int k = (int)op.targets.size(), D0 = 1 << k;
+    unsigned short *o = reinterpret_cast<unsigned short *>(out);
+    auto entry = [&](int r, int c) -> cd {  // group bits from k on: identity
+        if ((r >> k) != (c >> k)) return cd(0.0, 0.0);
+        return op.U[(size_t)(r & (D0 - 1)) * D0 + (c & (D0 - 1))];
+    };
+    const int tabs = C::TABS == 3 ? 2 : 1;
+    const double scale = std::ldexp(1.0, 62 - su);
+    unsigned short dg[kDigits];
+    for (int tab = 0; tab < tabs; tab++)
+        for (int mt = 0; mt < C::MT; mt++)
+            for (int ks = 0; ks < C::KS; ks++)
+                for (int lane = 0; lane < 32; lane++)
+                    for (int e = 0; e < 8; e++) {
+                        // A fragment half e: register e / 2 (row + 8 for 1, 3; column + 8 for 2, 3)
+                        const int row = (lane >> 2) + 8 * ((e >> 1) & 1);
+                        const int kp = 2 * (lane & 3) + (e & 1) + 8 * (e >> 2);
+                        double u;
+                        if (C::RF) {  // rows: re of amplitude 0..7, then im; columns: (re, im) pairs
+                            const cd z = entry(row & 7, kp >> 1);
+                            if (row < 8) u = (kp & 1) ? -z.imag() : z.real();
+                            else u = (kp & 1) ? z.real() : z.imag();
+                        } else {  // column kp: amplitude (q + 4 (e + 2 h)) of the k-step
+                            const int c = 16 * ks + ((kp & 7) >> 1) + 4 * ((kp & 1) + 2 * (kp >> 3));
+                            const cd z = entry(16 * mt + row, c);
+                            u = tab ? z.imag() : z.real();
+                        }
+                        digits_of(u, scale, dg);
+                        for (int j = 0; j < kDigits; j++)
+                            o[((((size_t)(tab * C::MT + mt) * C::KS + ks) * kDigits + j) * 32 + lane) * 8 + e] = dg[j];
+                    }
+}
+
+template <int K, bool REALU, int TBITS>
+static void launch(const Args &a, int sms, cudaStream_t st) {
+    using C = Cfg<K, REALU, TBITS>;
+    auto kern = dense_f64_kernel<K, REALU, TBITS>;
+    static bool attr = false;
+    if (!attr) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+        if (e != cudaSuccess) throw Error(QSIM_ECUDA, std::string("dense_f64_kernel attribute: ") + cudaGetErrorString(e));
+        attr = true;
+    }
+    const int per_sm = occupancy_cached(reinterpret_cast<const void *>(kern), C::THREADS, C::SMEM);
+    QSIM_REQUIRE(per_sm > 0, "dense_f64_kernel does not fit on an SM");
+    const int wpc = C::THREADS / 32;
+    const long long grid = std::min<long long>((a.ntasks + wpc - 1) / wpc, (long long)sms * per_sm);
+    kern<<<(int)grid, C::THREADS, C::SMEM, st>>>(a);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) throw Error(QSIM_ECUDA, std::string("dense_f64_kernel: ") + cudaGetErrorString(e));
+    note_launches(1, QSIM_KERNEL_DENSE_TC);
+}
+
+#define QSIM_F64_SWITCH(op, CALL)                            \
+    switch (f64::width_of(op) + (f64::real_form(op) ? 10 : 0)) { \
+        case 3: CALL(3, false); break;                       \
+        case 4: CALL(4, false); break;                       \
+        case 5: CALL(5, false); break;                       \
+        case 6: CALL(6, false); break;                       \
+        case 14: CALL(4, true); break;                       \
+        case 15: CALL(5, true); break;                       \
+        case 16: CALL(6, true); break;                       \
+        default: break;                                      \
+    }
+
+}  // namespace f64
+
+// Rows of U that are rows of the identity (their amplitudes do not change).
+static unsigned long long identity_rows(const Op &op) {
+    const int D = 1 << (int)op.targets.size();
+    unsigned long long keep = 0;
+    for (int r = 0; r < D; r++) {
+        bool id = true;
+        for (int c = 0; c < D && id; c++) id = op.U[(size_t)r * D + c] == cd(r == c ? 1.0 : 0.0, 0.0);
+        if (id) keep |= 1ull << r;
+    }
+    return keep;
+}
+
+// Gates of 1..6 targets whose rows are mostly nonzero.  A sum of a few terms that misses the group's
+// largest value is more exact in FP64 than relative to that value (a permutation is exact), so a
+// gate with a row of at most half its entries nonzero (identity rows and columns apart) stays plain.
+bool dense_f64_applies(const Op &op) {
+    const int k = (int)op.targets.size();
+    if (op.kind != OP_DENSE || k < 1 || k > 6) return false;
+    const int D = 1 << k;
+    const unsigned long long keep = identity_rows(op);
+    double top = 0.0;
+    int live = 0;
+    for (int r = 0; r < D; r++) live += !((keep >> r) & 1ull);
+    for (int r = 0; r < D; r++) {
+        if ((keep >> r) & 1ull) continue;
+        int nz = 0;
+        for (int c = 0; c < D; c++) {
+            const cd u = op.U[(size_t)r * D + c];
+            top = std::max(top, std::max(std::fabs(u.real()), std::fabs(u.imag())));
+            if (!((keep >> c) & 1ull)) nz += u != cd(0.0, 0.0);
+        }
+        if (2 * nz <= live) return false;
+    }
+    return live > 0 && top > std::ldexp(1.0, -100) && top < std::ldexp(1.0, 100);
+}
+
+size_t dense_f64_blob_bytes(const Op &op) {
+    size_t n = 0;
+#define QSIM_F64_BYTES(K, R) n = (size_t)f64::Cfg<K, R>::TAB * 16 * (f64::Cfg<K, R>::TABS == 3 ? 2 : 1)
+    QSIM_F64_SWITCH(op, QSIM_F64_BYTES)
+#undef QSIM_F64_BYTES
+    return n;
+}
+
+// exponent of U's scale: every entry is below 2^su in magnitude
+static int scale_of(const Op &op) {
+    double top = 0.0;
+    for (const cd &u : op.U) top = std::max(top, std::max(std::fabs(u.real()), std::fabs(u.imag())));
+    int e = 0;
+    std::frexp(top, &e);  // top = f 2^e, f in [1/2, 1)
+    return e;
+}
+
+void dense_f64_pack(Op &op, unsigned char *out) {
+    op.f64_su = scale_of(op);
+    op.f64_keep = identity_rows(op);
+#define QSIM_F64_PACK(K, R) f64::pack_digits<K, R>(op, op.f64_su, out)
+    QSIM_F64_SWITCH(op, QSIM_F64_PACK)
+#undef QSIM_F64_PACK
+}
+
+// Returns false when the state is too small for the kernel's tiles (the plain kernels take it).
+bool launch_dense_f64(void *state, int n, const Op &op, const void *dig, const void *Ut, int sms, cudaStream_t st) {
+    const int k = (int)op.targets.size(), K = f64::width_of(op);
+    int tb = 0, gb = 0, warps = 0;  // warps: of a full chip
+#define QSIM_F64_BITS(KK, R) tb = f64::Cfg<KK, R>::TB, gb = f64::Cfg<KK, R>::GB, warps = sms * f64::Cfg<KK, R>::THREADS / 32
+    QSIM_F64_SWITCH(op, QSIM_F64_BITS)
+#undef QSIM_F64_BITS
+    unsigned long long used = 0, cmask = 0;
+    for (int q : op.targets) used |= 1ull << q;
+    for (int q : op.controls) used |= 1ull << q, cmask |= 1ull << q;
+    std::vector<int> fr;  // free qubits ascending: columns, then the amplitude bits from k on, then tiles
+    for (int q = 0; q < n; q++)
+        if (!((used >> q) & 1ull)) fr.push_back(q);
+    const int groups = (int)fr.size() - gb - (K - k);  // tiles, log2
+    if (groups < tb || (1ll << (groups - tb)) < 2 * warps) tb = 0;
+    const int inside = gb + (K - k) + tb;
+    if ((int)fr.size() < inside || (int)(op.targets.size() + op.controls.size()) + inside > f64::kMaxFix) return false;
+    f64::Args a;
+    std::memset(&a, 0, sizeof(a));
+    a.psi = state;
+    a.dig = static_cast<const uint4 *>(dig);
+    a.Ut = static_cast<const double2 *>(Ut);
+    a.ntasks = 1ll << ((int)fr.size() - inside);
+    a.cmask = cmask;
+    a.su = op.f64_su;
+    a.k = k;
+    a.real_u = op.real_u ? 1 : 0;
+    for (int r = 0; r < (1 << K); r++)
+        if ((op.f64_keep >> (r & ((1 << k) - 1))) & 1ull) a.keep |= 1ull << r;
+    std::vector<int> amp(op.targets), fix(op.targets);
+    std::sort(amp.begin(), amp.end());
+    for (int j = 0; j < K - k; j++) amp.push_back(fr[gb + j]);
+    for (int v = 0; v < (1 << K); v++)
+        for (int b = 0; b < K; b++)
+            if ((v >> b) & 1) a.amp[v] += 16ll << amp[b];
+    for (int v = 0; v < (1 << gb); v++)
+        for (int b = 0; b < gb; b++)
+            if ((v >> b) & 1) a.col[v] += 16ll << fr[b];
+    for (int v = 0; v < (1 << tb); v++)
+        for (int b = 0; b < tb; b++)
+            if ((v >> b) & 1) a.tile[v] += 16ll << fr[gb + K - k + b];
+    fix.insert(fix.end(), op.controls.begin(), op.controls.end());
+    fix.insert(fix.end(), fr.begin(), fr.begin() + inside);
+    std::sort(fix.begin(), fix.end());
+    a.nfix = (int)fix.size();
+    for (int i = 0; i < a.nfix; i++) a.fix[i] = fix[i];
+#define QSIM_F64_LAUNCH(KK, R)                                                                  \
+    do {                                                                                        \
+        if (tb) f64::launch<KK, R, f64::Cfg<KK, R>::TBMAX>(a, sms, st);                         \
+        else f64::launch<KK, R, 0>(a, sms, st);                                                 \
+    } while (0)
+    QSIM_F64_SWITCH(op, QSIM_F64_LAUNCH)
+#undef QSIM_F64_LAUNCH
+    return true;
+}
+
+}  // namespace qsim

@@ -1136,6 +1136,15 @@ std::vector<unsigned char> pack_device_blob(qsim_circuit *c, int dtype) {
                 blob.resize(blob.size() + dense_tc_blob_bytes(6));
                 dense_tc_pack(6, UW, blob.data() + op.dev_off_tcw);
             }
+            if (dtype == QSIM_C128) {
+                op.has_f64 = dense_f64_applies(op);
+                if (op.has_f64) {
+                    align_blob(blob);
+                    op.dev_off_tc[slot] = blob.size();
+                    blob.resize(blob.size() + dense_f64_blob_bytes(op));
+                    dense_f64_pack(op, blob.data() + op.dev_off_tc[slot]);
+                }
+            }
             // the gate's own tensor-core form (also where the widened one is not taken)
             if (dtype == QSIM_C64 && dense_tc_supported((int)op.targets.size())) {
                 align_blob(blob);
@@ -1379,6 +1388,9 @@ void apply_ops(void *state, int n, int dtype, qsim_circuit *c, void *stream, int
                                               s7, n - 1, &sums_done))
                         break;
                 }
+                if (dtype == QSIM_C128 && op.has_f64 &&
+                    launch_dense_f64(state, w, op, base + op.dev_off_tc[slot], dptr, num_sms(), st))
+                    break;
                 run_dense(state, w, dtype, op, dptr, st);
                 break;
             case OP_PHASE: run_phase(state, w, dtype, op, st); break;
