@@ -218,6 +218,11 @@ void batch_enqueue_results(qsim_batch *b, cudaStream_t st);
 void batch_host_result(const qsim_batch *b, int i, double *x_out, hhl_readout_stats *stats);
 // dft.cu: Fourier-transform pass; tables packed into the circuit blob as W, Tlo, Thi
 void dft_tables(const Op &op, std::vector<cd> &W, std::vector<cd> &Tlo, std::vector<cd> &Thi);
+// dft_fx.cu: the same tables, and a structured phase's, as 60-bit integers in halves (4 ints per
+// entry), packed behind them for complex128
+int dft_table_split(int K, int ns);
+void dft_fixed_tables(const Op &op, std::vector<int> &out);
+void phase_fixed_table(const std::vector<cd> &v, std::vector<int> &out);
 // qop (OP_QPE_PHASE, optional): its diagonal applied to the pass's inputs (qmode 1) or outputs
 // (qmode 2), tables qlo / qhi as packed for that op
 // inv (OP_HHL_INVERT on qubit n, optional): applied to the outputs, which then also fill the

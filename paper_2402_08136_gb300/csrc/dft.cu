@@ -58,6 +58,7 @@ static bool dft_common_args(DftArgs &a, void *state, int n, int dtype, const Op 
     a.W = t;
     a.Tlo = t + vb * ((size_t)1 << K);
     a.Thi = t + vb * (((size_t)1 << K) + ((size_t)1 << hT));
+    a.Wfx = t + vb * (((size_t)1 << K) + ((size_t)1 << hT) + ((size_t)1 << (K + ns - hT)));
     a.hT = hT;
     a.ns = ns;
     a.twmode = ns == 0 ? 0 : (op.pre ? 1 : 2);
@@ -68,6 +69,7 @@ static bool dft_common_args(DftArgs &a, void *state, int n, int dtype, const Op 
         a.qnb = (int)qop->targets.size();
         a.qm = (int)qop->controls.size();
         a.qh = (a.qm + 1) / 2;  // the split qpe_phase_tables uses
+        a.qfx = static_cast<const unsigned char *>(qhi) + (vb << (a.qnb + a.qm - a.qh));
         bool contig_field = true;
         for (int j = 0; j < K; j++) contig_field = contig_field && op.targets[j] == op.targets[0] + j;
         // complex64 only: the recurrence rounds differently from the tables, which complex128's
@@ -169,6 +171,14 @@ bool run_dft(void *state, int n, int dtype, const Op &op, const void *tables, cu
     if (ns > 0 && smem + tw_bytes <= 200 * 1024) {
         a.tw_smem = 1;
         smem += tw_bytes;
+    }
+    if (dtype == QSIM_C128 && contig) {
+        DftArgs t = a;
+        t.inv_shared = a.inv;
+        for (int q : inv ? inv->controls : std::vector<int>())
+            for (int i = 0; i < L; i++)
+                if (a.lpos[i] == q) t.inv_shared = 0;
+        if (dft_launch_fx(t, K, op.sign, kind, st)) return true;
     }
     if (dtype == QSIM_C128) dft_launch_f64(a, K, op.sign, kind, contig, threads, smem, st);
     else dft_launch_f32(a, K, op.sign, kind, contig, threads, smem, st);

@@ -96,6 +96,10 @@ struct DftArgs {
     int inv, inv_bit, inv_twos, inv_nc, inv_fdst, inv_nseg;
     double inv_Cs;
     int inv_src[8], inv_w[8], inv_dst[8];
+    // complex128 fixed-point passes (dft_fx.cuh): the tables W, Tlo, Thi and qlo, qhi as integers;
+    // inv_shared: no lane qubit is a clock qubit of the inversion
+    const void *Wfx, *qfx;
+    int inv_shared;
     int fpos[kMaxK];            // qubit of field bit j
     int lpos[kMaxLane];         // qubit of lane bit j
     int spos[kMaxSrc];          // qubit of twiddle-source bit j
@@ -489,6 +493,9 @@ void launch_dtype(const DftArgs &a, int K, int sign, int kind, bool contig, int 
 }
 
 }  // namespace dftk
+
+// dft_fx.cu: complex128 pass on a contiguous field in fixed point; false when the shape does not fit
+bool dft_launch_fx(const dftk::DftArgs &a, int K, int sign, int kind, cudaStream_t st);
 
 // one per precision (dft_f32.cu, dft_f64.cu)
 void dft_launch_f32(const dftk::DftArgs &a, int K, int sign, int kind, bool contig, int threads, size_t smem,

@@ -783,6 +783,11 @@ void put_complex(std::vector<unsigned char> &blob, int dtype, const cd &z) {
     }
 }
 
+void put_ints(std::vector<unsigned char> &blob, const std::vector<int> &v) {
+    const unsigned char *p = reinterpret_cast<const unsigned char *>(v.data());
+    blob.insert(blob.end(), p, p + v.size() * sizeof(int));
+}
+
 void align_blob(std::vector<unsigned char> &blob) {
     while (blob.size() % 256) blob.push_back(0);
 }
@@ -1172,12 +1177,23 @@ std::vector<unsigned char> pack_device_blob(qsim_circuit *c, int dtype) {
             align_blob(blob);
             op.dev_off_tc[slot] = blob.size();  // second table
             for (const cd &z : hi) put_complex(blob, dtype, z);
+            if (dtype == QSIM_C128) {
+                std::vector<int> fixed;
+                phase_fixed_table(lo, fixed);
+                phase_fixed_table(hi, fixed);
+                put_ints(blob, fixed);
+            }
         } else if (op.kind == OP_DFT || op.kind == OP_WALSH) {
             std::vector<cd> W, Tlo, Thi;
             dft_tables(op, W, Tlo, Thi);
             for (const cd &z : W) put_complex(blob, dtype, z);
             for (const cd &z : Tlo) put_complex(blob, dtype, z);
             for (const cd &z : Thi) put_complex(blob, dtype, z);
+            if (dtype == QSIM_C128 && op.kind == OP_DFT) {
+                std::vector<int> fixed;
+                dft_fixed_tables(op, fixed);
+                put_ints(blob, fixed);
+            }
         }
     }
     align_blob(blob);
