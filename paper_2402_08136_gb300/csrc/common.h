@@ -104,11 +104,12 @@ struct Op {
     std::vector<int> tc_pads;
     size_t dev_off_tcw = 0;
     // complex128 dense op that runs as exact digit products on the tensor cores (dense_f64.cu; its
-    // digits at dev_off_tc[1]): entries of U are below 2^f64_su, bit r of f64_keep: row r is row r
-    // of the identity
+    // digits at dev_off_tc[1]): entries of U are below 2^f64_su, bit r of f64_diag: row and column r
+    // are zero off the diagonal
     bool has_f64 = false;
     int f64_su = 0;
-    unsigned long long f64_keep = 0;
+    unsigned long long f64_diag = 0;
+    int sparse_w = 0;  // complex128 dense op of at most this many nonzeros a row (dense_sparse.cu; entries at dev_off_tc[1])
     bool real_u = false;        // OP_DENSE: every entry of U is real (SIMT kernels use 2 FMAs per entry)
 };
 
@@ -200,9 +201,15 @@ bool launch_dense_tc_real7(void *state, int n, const std::vector<int> &targets, 
 // dense_f64.cu: complex128 dense gates as exact digit products on the tensor cores
 bool dense_f64_applies(const Op &op);
 size_t dense_f64_blob_bytes(const Op &op);
-void dense_f64_pack(Op &op, unsigned char *out);  // sets op.f64_su, op.f64_keep
+void dense_f64_pack(Op &op, unsigned char *out);  // sets op.f64_su, op.f64_diag
 // Ut: U in FP64, transposed; false (nothing launched) when the state has too few groups
 bool launch_dense_f64(void *state, int n, const Op &op, const void *dig, const void *Ut, int sms, cudaStream_t st);
+// dense_sparse.cu: complex128 gates whose rows are mostly zeros (sparse_width: entries a row, 0 if
+// not sparse); any gate of 3..7 targets on a state of at most 8 groups (false: more groups)
+int sparse_width(const Op &op);
+void sparse_pack(const Op &op, std::vector<unsigned char> &blob);
+void launch_sparse(void *state, int n, const Op &op, const void *ell, const void *Ut, int sms, cudaStream_t st);
+bool launch_group(void *state, int n, int dtype, const Op &op, const void *Ut, cudaStream_t st);
 // batched.cu: plan (host image) / instantiate (device tables) / launch / results, for the pool
 struct BatchImage;
 bool batch_supported(const qsim_circuit *c);  // every op runs in the batched executor
@@ -223,6 +230,10 @@ void dft_tables(const Op &op, std::vector<cd> &W, std::vector<cd> &Tlo, std::vec
 int dft_table_split(int K, int ns);
 void dft_fixed_tables(const Op &op, std::vector<int> &out);
 void phase_fixed_table(const std::vector<cd> &v, std::vector<int> &out);
+// complex128 broadcast of a pass on the field w .. w+K-1 still |0> (expand_kernel's outputs y >= 1) times
+// the structured phase of tables qlo, qhi (as packed for that op)
+void launch_expand_fx(void *state, int w, int K, double scale, const void *qlo, const void *qhi, int qnb, int qm, int qh,
+                      cudaStream_t st);
 // qop (OP_QPE_PHASE, optional): its diagonal applied to the pass's inputs (qmode 1) or outputs
 // (qmode 2), tables qlo / qhi as packed for that op
 // inv (OP_HHL_INVERT on qubit n, optional): applied to the outputs, which then also fill the

@@ -25,8 +25,9 @@
 // are output amplitudes, written back in place.  U's digits sit in shared memory in fragment order.
 // Group bits are the lowest free qubits, so a warp's load covers whole 128-byte lines.
 //
-// Not all gates take this form (dense_f64_applies): one whose rows are mostly zeros keeps the plain
-// kernel, which is exact on permutations; rows that are rows of the identity are not written at all.
+// Not all gates take this form (dense_f64_applies): one whose rows are mostly zeros keeps the FP64
+// kernels, which are exact on permutations; rows that only scale their own amplitude (the padding of
+// an eigenvector matrix, a controlled gate written as a dense one) are computed in FP64 on the way out.
 // A tile with a group that is not finite, or whose largest exponent is far from 1, is computed in
 // the plain FP64 form by the same warp (plain_tile).
 #include <cuda_runtime.h>
@@ -51,7 +52,7 @@ struct Args {
     const double2 *Ut;           // U transposed, FP64 (plain_tile)
     long long ntasks;
     unsigned long long cmask;
-    unsigned long long keep;     // bit r set: row r of U is row r of the identity (not written)
+    unsigned long long diag;     // bit r set: row and column r are zero off the diagonal (computed in FP64)
     int su;                      // U = (integers) 2^(su - 62)
     int k;                       // the gate's own targets (below 3: the rest of the 8 amplitudes are group bits)
     int real_u;
@@ -181,6 +182,23 @@ __device__ __noinline__ void plain_tile(const Args &a, char *base, int lane) {
         *reinterpret_cast<double2 *>(p + a.amp[lane % LPG + o * LPG]) = y[o];
     }
     __syncwarp();
+}
+
+// The result y of amplitude `row` into its place: for a diagonal row, U's entry times the value there.
+template <int K>
+__device__ __forceinline__ void put(const Args &a, int row, char *at, double2 y) {
+    double2 *p = reinterpret_cast<double2 *>(at);
+    if ((a.diag >> row) & 1ull) {
+        const int r = row & ((1 << a.k) - 1);
+        const double2 u = __ldg(a.Ut + (r << a.k) + r), x = *p;
+        y.x = u.x * x.x;
+        y.y = u.x * x.y;
+        if (!a.real_u) {
+            y.x = fma(-u.y, x.y, y.x);
+            y.y = fma(u.y, x.x, y.y);
+        }
+    }
+    __stcs(p, y);
 }
 
 template <int K, bool REALU, int TBITS>
@@ -327,8 +345,7 @@ __global__ void __launch_bounds__(Cfg<K, REALU>::THREADS, 1) dense_f64_kernel(co
 #pragma unroll
                 for (int j = 0; j < 2; j++) {  // amplitude n of group q + 4 j
                     const double2 y = make_double2(join<C>(acc[j], ex[j]), join<C>(acc[2 + j], ex[j]));
-                    if (!((a.keep >> n) & 1ull))
-                        __stcs(reinterpret_cast<double2 *>(ob + a.col[4 * j]), y);
+                    put<K>(a, n, ob + a.col[4 * j], y);
                 }
             } else {
 #pragma unroll 1
@@ -342,8 +359,7 @@ __global__ void __launch_bounds__(Cfg<K, REALU>::THREADS, 1) dense_f64_kernel(co
                         for (int h = 0; h < 2; h++) {  // amplitudes n and n + 8 of group q
                             const int row = 16 * mt + 8 * h + n;
                             const double2 y = make_double2(join<C>(acc[2 * h], ex[0]), join<C>(acc[2 * h + 1], ex[1]));
-                            if (!((a.keep >> row) & 1ull))
-                                __stcs(reinterpret_cast<double2 *>(ob + a.amp[16 * mt + 8 * h]), y);
+                            put<K>(a, row, ob + a.amp[16 * mt + 8 * h], y);
                         }
                     } else {
                         double re[4];
@@ -365,8 +381,7 @@ __global__ void __launch_bounds__(Cfg<K, REALU>::THREADS, 1) dense_f64_kernel(co
                         for (int c = 0; c < 4; c++) {  // amplitudes n and n + 8 of groups q and q + 4
                             const int row = 16 * mt + 8 * (c >> 1) + n;
                             const double2 y = make_double2(re[c], join<C>(acc[c], ex[c & 1]));
-                            if (!((a.keep >> row) & 1ull))
-                                __stcs(reinterpret_cast<double2 *>(ob + a.col[4 * (c & 1)] + a.amp[16 * mt + 8 * (c >> 1)]), y);
+                            put<K>(a, row, ob + a.col[4 * (c & 1)] + a.amp[16 * mt + 8 * (c >> 1)], y);
                         }
                     }
                 }
@@ -473,36 +488,37 @@ static void launch(const Args &a, int sms, cudaStream_t st) {
 
 }  // namespace f64
 
-// Rows of U that are rows of the identity (their amplitudes do not change).
-static unsigned long long identity_rows(const Op &op) {
+// Rows that, with their columns, are zero off the diagonal.
+static unsigned long long diagonal_rows(const Op &op) {
     const int D = 1 << (int)op.targets.size();
-    unsigned long long keep = 0;
+    unsigned long long diag = 0;
     for (int r = 0; r < D; r++) {
-        bool id = true;
-        for (int c = 0; c < D && id; c++) id = op.U[(size_t)r * D + c] == cd(r == c ? 1.0 : 0.0, 0.0);
-        if (id) keep |= 1ull << r;
+        bool d = true;
+        for (int c = 0; c < D && d; c++)
+            d = c == r || (op.U[(size_t)r * D + c] == cd(0.0, 0.0) && op.U[(size_t)c * D + r] == cd(0.0, 0.0));
+        if (d) diag |= 1ull << r;
     }
-    return keep;
+    return diag;
 }
 
 // Gates of 1..6 targets whose rows are mostly nonzero.  A sum of a few terms that misses the group's
 // largest value is more exact in FP64 than relative to that value (a permutation is exact), so a
-// gate with a row of at most half its entries nonzero (identity rows and columns apart) stays plain.
+// gate with a row of at most half its entries nonzero (diagonal rows and columns apart) stays in FP64.
 bool dense_f64_applies(const Op &op) {
     const int k = (int)op.targets.size();
     if (op.kind != OP_DENSE || k < 1 || k > 6) return false;
     const int D = 1 << k;
-    const unsigned long long keep = identity_rows(op);
+    const unsigned long long diag = diagonal_rows(op);
     double top = 0.0;
     int live = 0;
-    for (int r = 0; r < D; r++) live += !((keep >> r) & 1ull);
+    for (int r = 0; r < D; r++) live += !((diag >> r) & 1ull);
     for (int r = 0; r < D; r++) {
-        if ((keep >> r) & 1ull) continue;
+        if ((diag >> r) & 1ull) continue;
         int nz = 0;
         for (int c = 0; c < D; c++) {
             const cd u = op.U[(size_t)r * D + c];
             top = std::max(top, std::max(std::fabs(u.real()), std::fabs(u.imag())));
-            if (!((keep >> c) & 1ull)) nz += u != cd(0.0, 0.0);
+            if (!((diag >> c) & 1ull)) nz += u != cd(0.0, 0.0);
         }
         if (2 * nz <= live) return false;
     }
@@ -528,7 +544,7 @@ static int scale_of(const Op &op) {
 
 void dense_f64_pack(Op &op, unsigned char *out) {
     op.f64_su = scale_of(op);
-    op.f64_keep = identity_rows(op);
+    op.f64_diag = diagonal_rows(op);
 #define QSIM_F64_PACK(K, R) f64::pack_digits<K, R>(op, op.f64_su, out)
     QSIM_F64_SWITCH(op, QSIM_F64_PACK)
 #undef QSIM_F64_PACK
@@ -562,7 +578,7 @@ bool launch_dense_f64(void *state, int n, const Op &op, const void *dig, const v
     a.k = k;
     a.real_u = op.real_u ? 1 : 0;
     for (int r = 0; r < (1 << K); r++)
-        if ((op.f64_keep >> (r & ((1 << k) - 1))) & 1ull) a.keep |= 1ull << r;
+        if ((op.f64_diag >> (r & ((1 << k) - 1))) & 1ull) a.diag |= 1ull << r;
     std::vector<int> amp(op.targets), fix(op.targets);
     std::sort(amp.begin(), amp.end());
     for (int j = 0; j < K - k; j++) amp.push_back(fr[gb + j]);

@@ -1026,6 +1026,10 @@ void run_expand(void *state, int w, int dtype, const Op &op, const Op *qop, cons
     }
     for (int pass = 0; pass < 2; pass++) {  // outputs y >= 1 first, then column 0 in place
         a.col0 = pass;
+        if (!pass && dtype == QSIM_C128 && a.qmode == 2) {
+            launch_expand_fx(state, w, K, a.scale, qlo, qhi, a.qnb, a.qm, a.qh, st);
+            continue;
+        }
         const long long runs = (((1ll << K) - 1) + a.run - 1) / a.run;
         a.count = pass ? a.lowN : a.lowN * runs;
         const int grid = grid_for(a.count, 256);
@@ -1148,6 +1152,10 @@ std::vector<unsigned char> pack_device_blob(qsim_circuit *c, int dtype) {
                     op.dev_off_tc[slot] = blob.size();
                     blob.resize(blob.size() + dense_f64_blob_bytes(op));
                     dense_f64_pack(op, blob.data() + op.dev_off_tc[slot]);
+                } else if ((op.sparse_w = sparse_width(op)) > 0) {
+                    align_blob(blob);
+                    op.dev_off_tc[slot] = blob.size();
+                    sparse_pack(op, blob);
                 }
             }
             // the gate's own tensor-core form (also where the widened one is not taken)
@@ -1379,6 +1387,7 @@ void apply_ops(void *state, int n, int dtype, qsim_circuit *c, void *stream, int
         materialize(top_qubit(op) + 1);
         switch (op.kind) {
             case OP_DENSE:
+                if (dtype == QSIM_C64 && launch_group(state, w, dtype, op, dptr, st)) break;
                 if (dtype == QSIM_C64 && !op.tc_pads.empty()) {
                     // widened with identity qubits; all of them must lie inside the live width.  Gates
                     // of 1..3 targets are widened only on states larger than L2 (2^24 amplitudes),
@@ -1407,6 +1416,11 @@ void apply_ops(void *state, int n, int dtype, qsim_circuit *c, void *stream, int
                 if (dtype == QSIM_C128 && op.has_f64 &&
                     launch_dense_f64(state, w, op, base + op.dev_off_tc[slot], dptr, num_sms(), st))
                     break;
+                if (dtype == QSIM_C128 && op.sparse_w > 0) {
+                    launch_sparse(state, w, op, base + op.dev_off_tc[slot], dptr, num_sms(), st);
+                    break;
+                }
+                if (dtype == QSIM_C128 && launch_group(state, w, dtype, op, dptr, st)) break;
                 run_dense(state, w, dtype, op, dptr, st);
                 break;
             case OP_PHASE: run_phase(state, w, dtype, op, st); break;
