@@ -107,6 +107,7 @@ struct Op {
     // digits at dev_off_tc[1]): entries of U are below 2^f64_su, bit r of f64_diag: row and column r
     // are zero off the diagonal
     bool has_f64 = false;
+    bool f64_tc = false;  // ... with the digits laid out for tcgen05 (dense_f64_tc.cu)
     int f64_su = 0;
     unsigned long long f64_diag = 0;
     int sparse_w = 0;  // complex128 dense op of at most this many nonzeros a row (dense_sparse.cu; entries at dev_off_tc[1])
@@ -201,9 +202,18 @@ bool launch_dense_tc_real7(void *state, int n, const std::vector<int> &targets, 
 // dense_f64.cu: complex128 dense gates as exact digit products on the tensor cores
 bool dense_f64_applies(const Op &op);
 size_t dense_f64_blob_bytes(const Op &op);
-void dense_f64_pack(Op &op, unsigned char *out);  // sets op.f64_su, op.f64_diag
+void dense_f64_scale(Op &op);  // sets op.f64_su, op.f64_diag
+void dense_f64_pack(const Op &op, unsigned char *out);
 // Ut: U in FP64, transposed; false (nothing launched) when the state has too few groups
 bool launch_dense_f64(void *state, int n, const Op &op, const void *dig, const void *Ut, int sms, cudaStream_t st);
+// dense_f64_tc.cu: the same products with tcgen05 for wide gates (4 and 5 targets complex, 6 targets real or
+// complex) of circuits whose states fill the chip (blob_bytes 0: not one of them, dense_f64.cu takes it); the
+// launch is false when the (live) state is smaller than one tile of 128 or 64 groups
+size_t dense_f64_tc_blob_bytes(const Op &op, int n);
+void dense_f64_tc_pack(const Op &op, unsigned char *out);
+bool launch_dense_f64_tc(void *state, int n, const Op &op, const void *dig, const void *Ut, int sms, cudaStream_t st);
+unsigned dense_f64_read_error();
+void dense_f64_clear_error();
 // dense_sparse.cu: complex128 gates whose rows are mostly zeros (sparse_width: entries a row, 0 if
 // not sparse); any gate of 3..7 targets on a state of at most 8 groups (false: more groups)
 int sparse_width(const Op &op);

@@ -38,13 +38,12 @@
 #include <cstring>
 
 #include "common.h"
+#include "f64_digits.cuh"
 
 namespace qsim {
 namespace f64 {
 
 constexpr int kMaxFix = 40;
-constexpr int kDigits = 8;
-constexpr int kMinExp = 200, kMaxExp = 1900;  // biased exponents of a group's largest value that take the split
 
 struct Args {
     void *psi;
@@ -91,66 +90,6 @@ __device__ __forceinline__ void mma(float (&d)[4], const uint4 &a, unsigned b0, 
         "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
         : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
-}
-
-__device__ __forceinline__ unsigned mag_bits(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
-
-// x as a 62-bit integer relative to 2^(E + 1) (E: a biased exponent not below x's), plus 128 in
-// every byte: byte i is digit i + 128 of the signed base-256 form, -128 <= digit <= 127
-__device__ __forceinline__ unsigned long long fixed_bytes(double x, int E) {
-    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-    const int s = E - (int)((hi >> 20) & 0x7ffu);
-    const unsigned mh = (__funnelshift_l(lo, hi, 9) & 0x1fffffffu) | 0x20000000u;
-    unsigned long long v = ((unsigned long long)mh << 32) | (lo << 9);
-    asm("shr.u64 %0, %0, %1;" : "+l"(v) : "r"(s));  // 0 from 64 on
-    const long long sg = (long long)((int)hi >> 31);
-    return (v ^ (unsigned long long)sg) + (0x8080808080808080ull - (unsigned long long)sg);
-}
-
-// The digits of two reals as FP16 pairs: out[i] = (digit i of a, digit i of b), i = 0 the highest.
-// A byte under 0x64 is FP16 1024 + byte.
-__device__ __forceinline__ void digit_pairs(unsigned long long a, unsigned long long b, unsigned (&out)[kDigits]) {
-    const __half2 off = __floats2half2_rn(1152.f, 1152.f);
-#pragma unroll
-    for (int w = 0; w < 2; w++) {
-        const unsigned x = w ? (unsigned)a : (unsigned)(a >> 32), y = w ? (unsigned)b : (unsigned)(b >> 32);
-        const unsigned t[2] = {__byte_perm(x, y, 0x7362), __byte_perm(x, y, 0x5140)};  // bytes 2, 3 and 0, 1
-#pragma unroll
-        for (int i = 0; i < 4; i++) {  // digit 4 w + i is byte 3 - i of the word
-            const unsigned h = __byte_perm(t[i >> 1], 0x64646464u, (i & 1) ? 0x4140 : 0x4342);
-            const __half2 r = __hsub2(*reinterpret_cast<const __half2 *>(&h), off);
-            out[4 * w + i] = *reinterpret_cast<const unsigned *>(&r);
-        }
-    }
-}
-
-constexpr float kBiasF = 12582912.0f;  // 1.5 2^23: an FP32 sum started there has its integer in its low bits
-
-// sum_t acc[t] 2^(8 (7 - t)) / 2^SH, rounded to FP64, times 2^(ex - 1023) (0 for a zero sum)
-template <typename C>
-__device__ __forceinline__ double join(const float (&acc)[kDigits], int ex) {
-    long long T;
-    if constexpr (C::BIAS) {
-        int h[4];
-#pragma unroll
-        for (int p = 0; p < 4; p++)
-            h[p] = (int)((__float_as_uint(acc[2 * p]) << 8) + __float_as_uint(acc[2 * p + 1]) - 257u * 0x4B400000u +
-                         (p == 3 ? 1u << (C::SH - 1) : 0u));
-        T = (long long)h[2] * (1 << (16 - C::SH)) + (long long)(h[3] >> C::SH);
-        T += (long long)h[1] * (1 << (32 - C::SH));
-        T += (long long)((unsigned long long)(unsigned)(h[0] << (16 - C::SH)) << 32);
-    } else {
-        long long p[2];
-#pragma unroll
-        for (int w = 0; w < 2; w++) {
-            p[w] = (long long)__float2int_rn(acc[4 * w]) * (1 << 24) + (long long)__float2int_rn(acc[4 * w + 1]) * (1 << 16);
-            p[w] += (long long)__float2int_rn(acc[4 * w + 2]) * (1 << 8) + (long long)__float2int_rn(acc[4 * w + 3]);
-        }
-        T = (p[0] << (32 - C::SH)) + ((p[1] + (1 << (C::SH - 1))) >> C::SH);
-    }
-    const double d = (double)T;
-    const int hi = __double2hiint(d);
-    return __hiloint2double(hi ? hi + (ex << 20) : 0, __double2loint(d));
 }
 
 // One tile in the plain FP64 form, U's columns in order as the plain kernels add them.
@@ -344,7 +283,7 @@ __global__ void __launch_bounds__(Cfg<K, REALU>::THREADS, 1) dense_f64_kernel(co
                 step(tabs, br[0]);
 #pragma unroll
                 for (int j = 0; j < 2; j++) {  // amplitude n of group q + 4 j
-                    const double2 y = make_double2(join<C>(acc[j], ex[j]), join<C>(acc[2 + j], ex[j]));
+                    const double2 y = make_double2(join<C::BIAS, C::SH>(acc[j], ex[j]), join<C::BIAS, C::SH>(acc[2 + j], ex[j]));
                     put<K>(a, n, ob + a.col[4 * j], y);
                 }
             } else {
@@ -358,7 +297,7 @@ __global__ void __launch_bounds__(Cfg<K, REALU>::THREADS, 1) dense_f64_kernel(co
 #pragma unroll
                         for (int h = 0; h < 2; h++) {  // amplitudes n and n + 8 of group q
                             const int row = 16 * mt + 8 * h + n;
-                            const double2 y = make_double2(join<C>(acc[2 * h], ex[0]), join<C>(acc[2 * h + 1], ex[1]));
+                            const double2 y = make_double2(join<C::BIAS, C::SH>(acc[2 * h], ex[0]), join<C::BIAS, C::SH>(acc[2 * h + 1], ex[1]));
                             put<K>(a, row, ob + a.amp[16 * mt + 8 * h], y);
                         }
                     } else {
@@ -370,7 +309,7 @@ __global__ void __launch_bounds__(Cfg<K, REALU>::THREADS, 1) dense_f64_kernel(co
                             step(tu + 2 * C::TAB + s * kDigits * 32, bi[s]);
                         }
 #pragma unroll
-                        for (int c = 0; c < 4; c++) re[c] = join<C>(acc[c], ex[c & 1]);
+                        for (int c = 0; c < 4; c++) re[c] = join<C::BIAS, C::SH>(acc[c], ex[c & 1]);
                         clear();
 #pragma unroll
                         for (int s = 0; s < KS; s++) {
@@ -380,34 +319,13 @@ __global__ void __launch_bounds__(Cfg<K, REALU>::THREADS, 1) dense_f64_kernel(co
 #pragma unroll
                         for (int c = 0; c < 4; c++) {  // amplitudes n and n + 8 of groups q and q + 4
                             const int row = 16 * mt + 8 * (c >> 1) + n;
-                            const double2 y = make_double2(re[c], join<C>(acc[c], ex[c & 1]));
+                            const double2 y = make_double2(re[c], join<C::BIAS, C::SH>(acc[c], ex[c & 1]));
                             put<K>(a, row, ob + a.col[4 * (c & 1)] + a.amp[16 * mt + 8 * (c >> 1)], y);
                         }
                     }
                 }
             }
         }
-    }
-}
-
-// u / 2^(su - 62) as signed base-256 digits, -127 <= digit <= 128 (so that no product of a digit
-// with one of the state's reaches +2^14), highest first, as FP16 bit patterns
-static void digits_of(double u, double scale, unsigned short (&d)[kDigits]) {
-    struct Half {
-        unsigned short bits[256];
-        Half() {
-            for (int v = 0; v < 256; v++) {
-                const __half h = __float2half_rn((float)(v - 127));
-                std::memcpy(&bits[v], &h, 2);
-            }
-        }
-    };
-    static const Half half;
-    long long w = std::llrint(u * scale);  // at most 2^62
-    for (int i = kDigits - 1; i >= 0; i--) {
-        const int b = (int)((w + 127) & 255);
-        d[i] = half.bits[b];
-        w = (w + 127 - b) / 256;
     }
 }
 
@@ -429,7 +347,6 @@ static void pack_digits(const Op &op, int su, unsigned char *out) {
     };
     const int tabs = C::TABS == 3 ? 2 : 1;
     const double scale = std::ldexp(1.0, 62 - su);
-    unsigned short dg[kDigits];
     for (int tab = 0; tab < tabs; tab++)
         for (int mt = 0; mt < C::MT; mt++)
             for (int ks = 0; ks < C::KS; ks++)
@@ -448,9 +365,9 @@ static void pack_digits(const Op &op, int su, unsigned char *out) {
                             const cd z = entry(16 * mt + row, c);
                             u = tab ? z.imag() : z.real();
                         }
-                        digits_of(u, scale, dg);
+                        const unsigned long long dg = digit_bytes(u, scale);
                         for (int j = 0; j < kDigits; j++)
-                            o[((((size_t)(tab * C::MT + mt) * C::KS + ks) * kDigits + j) * 32 + lane) * 8 + e] = dg[j];
+                            o[((((size_t)(tab * C::MT + mt) * C::KS + ks) * kDigits + j) * 32 + lane) * 8 + e] = half_digit(dg, j);
                     }
 }
 
@@ -542,9 +459,12 @@ static int scale_of(const Op &op) {
     return e;
 }
 
-void dense_f64_pack(Op &op, unsigned char *out) {
+void dense_f64_scale(Op &op) {
     op.f64_su = scale_of(op);
     op.f64_diag = diagonal_rows(op);
+}
+
+void dense_f64_pack(const Op &op, unsigned char *out) {
 #define QSIM_F64_PACK(K, R) f64::pack_digits<K, R>(op, op.f64_su, out)
     QSIM_F64_SWITCH(op, QSIM_F64_PACK)
 #undef QSIM_F64_PACK

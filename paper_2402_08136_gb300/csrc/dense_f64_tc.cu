@@ -1,0 +1,633 @@
+// Wide complex128 gates as exact digit products on the 5th-generation tensor cores (sm_103a):
+// tcgen05.mma kind::f16, eight FP32 accumulators per output in tensor memory.
+//
+// The digits and sums are dense_f64.cu's (see there for the split and its error).  Its warp-level MMAs run at
+// 1024 products per clock and SM, which bounds gates of 4 targets and more (36 2^(k+1) products a real);
+// tcgen05 runs four times as fast, and the accumulators leave the registers.
+//
+// A tile is 128 rows: 128 groups of a complex gate of 4 or 5 targets (a row holds the group's reals), or 64
+// groups times {re, im} of a 6-target gate.  Digit i of the rows is one MMA operand (A, 128 x 16 per K-step), and
+// the digits 0..7-i of U, stacked along N, are the other one: with accumulator t for the digit pairs i + j = t in
+// columns 32 t .. 32 t + 31, one MMA of N = 32 (8 - i) columns adds digit i's products with all of them to
+// accumulators i..7, and a K-step is 8 MMAs.  A unit is 32 output reals of a row, 256 columns; two units
+// alternate, so the sums of one are put together while the MMAs fill the other.
+//   4 targets            K = 32 reals,  1 unit
+//   5 targets            K = 64,        2 units (the rows' digits stay in shared memory for the second)
+//   6 targets, real U    K = 64,        2 units (rows (group, re or im))
+//   6 targets            K = 128: the row's own part times Re U, then the other part (negated for re) times
+//                        Im U; 2 units at once (U's digits leave room for two K-steps only)
+//
+// 17 warps: 8 load amplitudes (each thread 8 or 16 of them, the next tile's into the same registers as they are
+// used up), write their digits to a ring of K-steps and release it; one lane issues the MMAs; 8 read finished
+// units, put the sums together, and pass the amplitudes through shared memory so that a warp's store covers
+// 4 amplitudes of 8 groups (the lowest targets and free qubits: whole lines).  Roles meet at mbarriers only,
+// every wait is bounded, tensor memory is freed after the last MMA has completed (as in dense_tc.cu).
+// A tile with a group outside the fixed-point range is computed in FP64 by the reading warps (plain_tile).
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+
+#include "common.h"
+#include "f64_digits.cuh"
+#include "tc_ptx.cuh"
+
+namespace qsim {
+
+__device__ unsigned int g_f64_error = 0;
+
+namespace f64tc {
+
+using namespace f64;
+using namespace tc;
+
+constexpr int kMaxFix = 40;
+constexpr int kProdWarps = 8, kEpiWarps = 8, kMmaWarp = kProdWarps + kEpiWarps;
+constexpr int kThreads = (kMmaWarp + 4) * 32;  // the issuing warp's group of four is filled up for setmaxnreg
+// registers a thread: launched with 96 (640 threads), 61440 in all; 256 x 128 + 256 x 80 + 128 x 56 = 60416 after the split
+constexpr int kProdRegs = 128, kEpiRegs = 80, kMmaRegs = 56;
+constexpr int kSlot = kDigits * 4096;  // one K-step of a tile: 8 digits x 128 rows x 16 FP16
+constexpr int kBlock = 8192;           // U's digits of one unit and K-step: 256 rows x 16 FP16
+
+enum Mode { C4 = 0, C5 = 1, R6 = 2, C6 = 3 };
+
+template <int MODE>
+struct Cfg {
+    static constexpr int K = MODE == C4 ? 4 : MODE == C5 ? 5 : 6, D = 1 << K;
+    static constexpr bool PARTS = MODE >= R6;             // rows are (group, re or im)
+    static constexpr int GB = PARTS ? 6 : 7;              // group bits of a tile
+    static constexpr int KS = MODE == C4 ? 2 : MODE == C6 ? 8 : 4;  // K-steps
+    static constexpr int UNITS = MODE == C4 ? 1 : 2;
+    static constexpr int SLOTS = MODE == C6 ? 2 : 4;
+    static constexpr int ITEMS = PARTS ? 1 : 2;           // rows per loading thread
+    static constexpr int EPT = MODE == C4 ? 4 : MODE == C5 ? 8 : 16;  // amplitudes per item: every fourth
+    static constexpr int STEP = PARTS ? 4 : 2;            // amplitudes per item and K-step
+    static constexpr int RED = MODE == C4 ? 32 : MODE == C6 ? 128 : 64;
+    static constexpr bool BIAS = RED <= 32;
+    static constexpr int SH = RED > 64 ? 13 : 12;
+    static constexpr int BBYTES = UNITS * KS * kBlock;
+    static constexpr int STAGE = kEpiWarps * 2048;
+    static constexpr int SMEM = BBYTES + SLOTS * kSlot + STAGE + 4 * 128 * 4 + 16 + 8 * (2 * SLOTS + 5) + 16;
+};
+
+struct Args {
+    double2 *psi;
+    const uint4 *dig;
+    const double2 *Ut;
+    long long ntiles;
+    unsigned long long cmask, diag;
+    int su, nfix;
+    int fix[kMaxFix];   // ascending: targets, controls, group bits inside a tile
+    long long amp[64];  // offset (in amplitudes) of amplitude a of a group
+    long long grp[7];   // ... of group bit b of a tile
+};
+
+__device__ __forceinline__ void mma_f16(unsigned d, uint64_t adesc, uint64_t bdesc, unsigned idesc, unsigned accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+__device__ __forceinline__ void tmem_ld4(unsigned addr, float (&v)[4]) {
+    unsigned r[4];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr));
+#pragma unroll
+    for (int i = 0; i < 4; i++) v[i] = __uint_as_float(r[i]);
+}
+
+// A tile in FP64 by the 256 reading threads, U's columns in the plain kernels' order: all outputs before any store.
+template <int MODE>
+__device__ __noinline__ void plain_tile(const Args &a, double2 *base, int t) {
+    using C = Cfg<MODE>;
+    constexpr int D = C::D, TPG = 256 >> C::GB, OUT = D / TPG;  // threads per group, outputs per thread
+    const int g = t & ((1 << C::GB) - 1), part = t >> C::GB;
+    for (int b = 0; b < C::GB; b++)
+        if ((g >> b) & 1) base += a.grp[b];
+    double2 y[OUT];
+#pragma unroll 1
+    for (int o = 0; o < OUT; o++) {
+        const int r = part * OUT + o;
+        double2 s = make_double2(0.0, 0.0);
+#pragma unroll 1
+        for (int c = 0; c < D; c++) {
+            const double2 x = base[a.amp[c]], u = a.Ut[c * D + r];
+            s.x = fma(u.x, x.x, s.x);
+            if (MODE != R6) s.x = fma(-u.y, x.y, s.x);
+            s.y = fma(u.x, x.y, s.y);
+            if (MODE != R6) s.y = fma(u.y, x.x, s.y);
+        }
+        y[o] = s;
+    }
+    asm volatile("bar.sync 1, 256;\n" ::: "memory");
+#pragma unroll 1
+    for (int o = 0; o < OUT; o++) base[a.amp[part * OUT + o]] = y[o];
+}
+
+// z, or for a row that only scales its amplitude the value at p scaled.
+template <int MODE>
+__device__ __noinline__ double2 scaled_row(const Args &a, int row, const double2 *p, double2 z) {
+    if ((a.diag >> row) & 1ull) {
+        const double2 w = __ldg(a.Ut + row * Cfg<MODE>::D + row), o = *p;
+        z.x = w.x * o.x;
+        z.y = w.x * o.y;
+        if (MODE != R6) {
+            z.x = fma(-w.y, o.y, z.x);
+            z.y = fma(w.y, o.x, z.y);
+        }
+    }
+    return z;
+}
+// The amplitudes of 8 columns from the warp's stage to their places: lane (4 lowest amplitudes, 8 groups).
+template <int MODE, bool DIAG>
+__device__ __forceinline__ void store_body(const Args &a, const unsigned char *st, double2 *at, int h, int s, int lane) {
+    using C = Cfg<MODE>;
+    const int sa = lane & 3, sr = lane >> 2;
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        double2 z, *p = at;
+        int row;
+        if (C::PARTS) {
+            const int g = 8 * (i & 1) + sr, c = sa + 4 * (i >> 1);
+            z = *reinterpret_cast<const double2 *>(st + g * 128 + ((c ^ (g & 7)) * 16));
+            row = 32 * h + 8 * s + c;
+            p += ((i & 1) ? a.grp[3] : 0) + a.amp[32 * h + 8 * s + 4 * (i >> 1)];
+        } else {
+            const int r = 8 * i + sr;
+            z = *reinterpret_cast<const double2 *>(st + r * 64 + ((sa ^ ((r >> 1) & 3)) * 16));
+            row = 16 * h + 4 * s + sa;
+            p += ((i & 1) ? a.grp[3] : 0) + ((i & 2) ? a.grp[4] : 0) + a.amp[16 * h + 4 * s];
+        }
+        if (DIAG) z = scaled_row<MODE>(a, row, p, z);
+        __stcs(p, z);
+    }
+}
+template <int MODE>
+__device__ __noinline__ void store_diag(const Args &a, const unsigned char *st, double2 *at, int h, int s, int lane) {
+    store_body<MODE, true>(a, st, at, h, s, lane);
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_constant__ Args a) {
+    using C = Cfg<MODE>;
+    constexpr int KS = C::KS, SLOTS = C::SLOTS, ITEMS = C::ITEMS, EPT = C::EPT, STEP = C::STEP, UNITS = C::UNITS;
+    constexpr bool PARTS = C::PARTS;
+    extern __shared__ __align__(1024) unsigned char sm[];
+    unsigned char *ring = sm + C::BBYTES;
+    unsigned char *stage = ring + SLOTS * kSlot;
+    int *exps = reinterpret_cast<int *>(stage + C::STAGE);  // [4 tiles][128 rows]
+    int *odd = exps + 4 * 128;                              // [4 tiles]: the tile takes plain_tile
+    uint64_t *full = reinterpret_cast<uint64_t *>(odd + 4);
+    uint64_t *empty = full + SLOTS, *accfull = empty + SLOTS, *accempty = accfull + 2, *drain = accempty + 2;
+    unsigned *tslot = reinterpret_cast<unsigned *>(drain + 1);
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    for (int i = tid; i < C::BBYTES / 16; i += kThreads) reinterpret_cast<uint4 *>(sm)[i] = a.dig[i];
+    if (tid < 4) odd[tid] = 0;
+    if (tid == 0) {
+        for (int i = 0; i < SLOTS; i++) {
+            mbar_init(&full[i], kProdWarps);
+            mbar_init(&empty[i], 1);
+        }
+        for (int i = 0; i < 2; i++) {
+            mbar_init(&accfull[i], 1);
+            mbar_init(&accempty[i], kEpiWarps);
+        }
+        mbar_init(drain, 1);
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tslot)), "r"(512u)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    }
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    const unsigned tmem = *tslot;
+    const long long first = blockIdx.x, stride = gridDim.x;
+    const long long ntl = first < a.ntiles ? (a.ntiles - first + stride - 1) / stride : 0;
+    bool failed = false;
+    auto tile_base = [&](long long i) -> double2 * {
+        return a.psi + (insert_zeros((unsigned long long)(first + i * stride), a.fix, a.nfix) | a.cmask);
+    };
+
+    if (warp < kProdWarps) {
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(kProdRegs));
+        // ------------------------------------------------------------------ loads and digits
+        // Lane (r8, kc): row (group) 8 warp + r8 of every item, amplitudes kc + 4 e.  A load covers the 4 lowest
+        // amplitudes of 8 neighbouring groups.  K position of a thread's reals in a K-step: 4 kc ..
+        const int r8 = lane & 7, kc = lane >> 3;
+        long long off = a.amp[kc];
+#pragma unroll
+        for (int b = 0; b < 3; b++)
+            if ((r8 >> b) & 1) off += a.grp[b];
+#pragma unroll
+        for (int b = 0; b < 3; b++)
+            if ((warp >> b) & 1) off += a.grp[3 + b];
+        double2 x[ITEMS][EPT];
+        {
+            const double2 *p = tile_base(0) + off;
+#pragma unroll
+            for (int it = 0; it < ITEMS; it++)
+#pragma unroll
+                for (int e = 0; e < EPT; e++)
+                    if (ntl > 0) x[it][e] = __ldcs(p + (it ? a.grp[6] : 0) + a.amp[4 * e]);
+        }
+        const unsigned col = (unsigned)((kc >> 1) * 128 + (kc & 1) * 8);
+        for (long long t = 0; t < ntl && !failed; t++) {
+            int Er[ITEMS], Ei[ITEMS];
+#pragma unroll
+            for (int it = 0; it < ITEMS; it++) {
+                unsigned mr = 0, mi = 0, low = 0;
+#pragma unroll
+                for (int e = 0; e < EPT; e++) {
+                    mr = max(mr, mag_bits(x[it][e].x));
+                    mi = max(mi, mag_bits(x[it][e].y));
+                }
+                if (MODE != R6) mr = mi = max(mr, mi);  // one exponent for both parts where they mix
+                mr = max(mr, __shfl_xor_sync(~0u, mr, 8));
+                mr = max(mr, __shfl_xor_sync(~0u, mr, 16));
+                if (MODE == R6) {
+                    mi = max(mi, __shfl_xor_sync(~0u, mi, 8));
+                    mi = max(mi, __shfl_xor_sync(~0u, mi, 16));
+                } else {
+                    mi = mr;
+                }
+                Er[it] = mr ? (int)(mr >> 20) : 1023;
+                Ei[it] = mi ? (int)(mi >> 20) : 1023;
+                if (mr == 0 || mi == 0)  // all zero, or denormals whose high words are 0
+#pragma unroll
+                    for (int e = 0; e < EPT; e++) {
+                        if (!mag_bits(x[it][e].x)) low |= (unsigned)__double2loint(x[it][e].x);
+                        if (!mag_bits(x[it][e].y)) low |= (unsigned)__double2loint(x[it][e].y);
+                    }
+                if (Er[it] < kMinExp || Er[it] > kMaxExp || Ei[it] < kMinExp || Ei[it] > kMaxExp || low) odd[t & 3] = 1;
+                if (kc == 0) {
+                    int *ex = exps + (t & 3) * 128;
+                    if (PARTS) {
+                        ex[2 * (8 * warp + r8)] = Er[it];
+                        ex[2 * (8 * warp + r8) + 1] = Ei[it];
+                    } else {
+                        ex[64 * it + 8 * warp + r8] = Er[it];
+                    }
+                }
+            }
+            const bool more = t + 1 < ntl;
+            const double2 *np = tile_base(more ? t + 1 : t) + off;
+#pragma unroll
+            for (int s = 0; s < EPT / STEP; s++) {
+                constexpr int PER = MODE == C6 ? 2 : 1;  // slots per step
+                const long long q0 = (t * (EPT / STEP) + s) * PER;
+                auto wait_slot = [&](long long q) {  // the warp gives up together
+                    const bool ok = q < SLOTS || mbar_wait(&empty[q % SLOTS], (unsigned)((q / SLOTS - 1) & 1));
+                    if (!__all_sync(~0u, ok)) failed = true;
+                };
+                wait_slot(q0);
+                if (failed) break;
+                unsigned char *sl = ring + (q0 % SLOTS) * kSlot + col;
+                unsigned re[2][kDigits], im[2][kDigits];
+#pragma unroll
+                for (int it = 0; it < ITEMS; it++) {
+                    if constexpr (PARTS) {
+                        const double2 *v = x[it] + STEP * s;
+                        digit_pairs(fixed_bytes(v[0].x, Er[it]), fixed_bytes(v[1].x, Er[it]), re[0]);
+                        digit_pairs(fixed_bytes(v[2].x, Er[it]), fixed_bytes(v[3].x, Er[it]), re[1]);
+                        digit_pairs(fixed_bytes(v[0].y, Ei[it]), fixed_bytes(v[1].y, Ei[it]), im[0]);
+                        digit_pairs(fixed_bytes(v[2].y, Ei[it]), fixed_bytes(v[3].y, Ei[it]), im[1]);
+                        const int g = 8 * warp + r8;
+                        // rows 2 g and 2 g + 1, the order alternating so that 16 lanes fill distinct banks
+                        const int r0 = 2 * g + (r8 >> 2), r1 = r0 ^ 1;
+                        const unsigned o0 = (r0 >> 3) * 256 + (r0 & 7) * 16, o1 = (r1 >> 3) * 256 + (r1 & 7) * 16;
+#pragma unroll
+                        for (int d = 0; d < kDigits; d++) {
+                            const uint2 vr = make_uint2(re[0][d], re[1][d]), vi = make_uint2(im[0][d], im[1][d]);
+                            *reinterpret_cast<uint2 *>(sl + d * 4096 + o0) = (r8 >> 2) ? vi : vr;
+                            *reinterpret_cast<uint2 *>(sl + d * 4096 + o1) = (r8 >> 2) ? vr : vi;
+                        }
+                        if constexpr (MODE == C6) {
+                            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(&full[q0 % SLOTS]);
+                            wait_slot(q0 + 1);
+                            sl = ring + ((q0 + 1) % SLOTS) * kSlot + col;
+#pragma unroll
+                            for (int d = 0; d < kDigits; d++) {  // -im in the re row, re in the im row
+                                const uint2 vr = make_uint2(im[0][d] ^ 0x80008000u, im[1][d] ^ 0x80008000u);
+                                const uint2 vi = make_uint2(re[0][d], re[1][d]);
+                                *reinterpret_cast<uint2 *>(sl + d * 4096 + o0) = (r8 >> 2) ? vi : vr;
+                                *reinterpret_cast<uint2 *>(sl + d * 4096 + o1) = (r8 >> 2) ? vr : vi;
+                            }
+                        }
+                    } else {
+                        const double2 *v = x[it] + STEP * s;
+                        digit_pairs(fixed_bytes(v[0].x, Er[it]), fixed_bytes(v[0].y, Er[it]), re[0]);
+                        digit_pairs(fixed_bytes(v[1].x, Er[it]), fixed_bytes(v[1].y, Er[it]), re[1]);
+                        const int row = 64 * it + 8 * warp + r8;
+                        unsigned char *p = sl + (row >> 3) * 256 + (row & 7) * 16;
+#pragma unroll
+                        for (int d = 0; d < kDigits; d++)
+                            *reinterpret_cast<uint2 *>(p + d * 4096) = make_uint2(re[0][d], re[1][d]);
+                    }
+                    if (more)
+#pragma unroll
+                        for (int e = STEP * s; e < STEP * s + STEP; e++)
+                            x[it][e] = __ldcs(np + (it ? a.grp[6] : 0) + a.amp[4 * e]);
+                }
+                if (failed) break;
+                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&full[(q0 + PER - 1) % SLOTS]);
+            }
+        }
+    } else if (warp < kMmaWarp) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(kEpiRegs));
+        // ------------------------------------------------------------------ sums and stores
+        const int ew = warp - kProdWarps, sub = ew & 3;  // TMEM lanes 32 sub .. (warp mod 4 == sub)
+        const int m = 32 * sub + lane;                   // row
+        unsigned char *st = stage + ew * 2048;
+        // place in a store: 4 lowest amplitudes x 8 groups
+        const int sa = lane & 3, sr = lane >> 2;
+        long long off = a.amp[sa];
+#pragma unroll
+        for (int b = 0; b < 3; b++)
+            if ((sr >> b) & 1) off += a.grp[b];
+        off += (sub & 1) ? a.grp[PARTS ? 4 : 5] : 0;
+        off += (sub & 2) ? a.grp[PARTS ? 5 : 6] : 0;
+        for (long long u = 0; u < ntl * UNITS && !failed; u++) {
+            const long long t = u / UNITS;
+            const int h = (int)(u % UNITS), ab = (int)(u & 1);
+            bool ok = mbar_wait(&accfull[ab], (unsigned)((u >> 1) & 1));
+            ok = __all_sync(~0u, ok);
+            if (!ok) {
+                failed = true;
+                break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            double2 *base = tile_base(t);
+            const int ex = exps[(t & 3) * 128 + m] - 1022 + a.su - (68 - C::SH);
+            const bool plain = odd[t & 3] != 0;
+            if (plain && h == 0) plain_tile<MODE>(a, base, ew * 32 + lane);
+            const unsigned acc = tmem + (unsigned)(ab * 256) + ((unsigned)(32 * sub) << 16);
+            if (!plain) {
+#pragma unroll 1
+                for (int s = 2 * (ew >> 2); s < 2 * (ew >> 2) + 2; s++) {  // columns 8 s .. 8 s + 7 of the unit
+                    __syncwarp();  // the previous step's amplitudes have been read
+#pragma unroll
+                    for (int c4 = 0; c4 < 8; c4 += 4) {  // four columns at a time: 32 registers of sums
+                        float v[kDigits][4];
+#pragma unroll
+                        for (int d = 0; d < kDigits; d++) tmem_ld4(acc + (unsigned)(32 * d + 8 * s + c4), v[d]);
+                        asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+                        double y[4];
+#pragma unroll
+                        for (int c = 0; c < 4; c++) {
+                            float w[kDigits];
+#pragma unroll
+                            for (int d = 0; d < kDigits; d++) w[d] = C::BIAS ? v[d][c] + kBiasF : v[d][c];
+                            y[c] = join<C::BIAS, C::SH>(w, ex);
+                        }
+                        if (PARTS) {  // row (group, part): parts of 8 amplitudes
+                            const int g = lane >> 1;
+#pragma unroll
+                            for (int c = 0; c < 4; c++)
+                                *reinterpret_cast<double *>(st + g * 128 + (((c4 + c) ^ (g & 7)) * 16) + (lane & 1) * 8) = y[c];
+                        } else {      // row: 4 amplitudes
+#pragma unroll
+                            for (int c = 0; c < 2; c++)
+                                *reinterpret_cast<double2 *>(st + lane * 64 + (((c4 / 2 + c) ^ ((lane >> 1) & 3)) * 16)) =
+                                    make_double2(y[2 * c], y[2 * c + 1]);
+                        }
+                    }
+                    __syncwarp();
+                    // gates with rows that only scale their amplitude take a function of their own: as a condition
+                    // here its FP64 operations are predicated and pass through the FP64 pipe for every amplitude
+                    if (a.diag) store_diag<MODE>(a, st, base + off, h, s, lane);
+                    else store_body<MODE, false>(a, st, base + off, h, s, lane);
+                }
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+            if (h == UNITS - 1) {
+                // every reading warp is past its look at the tile's flag before it is taken back
+                asm volatile("bar.sync 1, 256;\n" ::: "memory");
+                if (ew == 0 && lane == 0) odd[t & 3] = 0;
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&accempty[ab]);
+        }
+    } else {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(kMmaRegs));
+        if (warp == kMmaWarp && lane == 0) {
+        // ------------------------------------------------------------------ MMAs
+        const unsigned b0 = smem_u32(sm), a0 = smem_u32(ring);
+        constexpr unsigned IDESC = (1u << 4) | ((unsigned)(128 >> 4) << 24);  // FP32 += FP16 x FP16, M = 128
+        auto kstep = [&](int slot, int h, int ks, int ab) {
+            const unsigned as = a0 + slot * kSlot, bs = b0 + (unsigned)((h * KS + ks) * kBlock);
+            const uint64_t ad = make_desc(as, 128, 256), bd = make_desc(bs, 128, 256);
+#pragma unroll
+            for (int i = 0; i < kDigits; i++)
+                mma_f16(tmem + (unsigned)(ab * 256 + 32 * i), ad + (uint64_t)(i * 4096 >> 4), bd,
+                        IDESC | ((unsigned)(32 * (kDigits - i) >> 3) << 17), (ks == 0 && i == 0) ? 0u : 1u);
+        };
+        auto free_unit = [&](long long u) {  // the unit's accumulators have been read
+            return u < 2 || mbar_wait(&accempty[u & 1], (unsigned)(((u >> 1) - 1) & 1));
+        };
+        for (long long t = 0; t < ntl && !failed; t++) {
+            if constexpr (MODE == C6) {
+                if (!free_unit(2 * t)) failed = true;
+#pragma unroll 1
+                for (int ks = 0; ks < KS && !failed; ks++) {
+                    const long long q = t * KS + ks;
+                    if (!mbar_wait(&full[q % SLOTS], (unsigned)((q / SLOTS) & 1))) {
+                        failed = true;
+                        break;
+                    }
+                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                    kstep((int)(q % SLOTS), 0, ks, 0);
+                    if (ks == 0 && !free_unit(2 * t + 1)) {
+                        failed = true;
+                        break;
+                    }
+                    kstep((int)(q % SLOTS), 1, ks, 1);
+                    commit_to(&empty[q % SLOTS]);
+                }
+                if (!failed) {
+                    commit_to(&accfull[0]);
+                    commit_to(&accfull[1]);
+                }
+            } else {
+#pragma unroll 1
+                for (int h = 0; h < UNITS && !failed; h++) {
+                    const long long u = t * UNITS + h;
+                    if (!free_unit(u)) failed = true;
+#pragma unroll 1
+                    for (int ks = 0; ks < KS && !failed; ks++) {
+                        const long long q = t * KS + ks;
+                        if (h == 0 && !mbar_wait(&full[q % SLOTS], (unsigned)((q / SLOTS) & 1))) {
+                            failed = true;
+                            break;
+                        }
+                        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                        kstep((int)(q % SLOTS), h, ks, (int)(u & 1));
+                        if (h == UNITS - 1) commit_to(&empty[q % SLOTS]);
+                    }
+                    if (!failed) commit_to(&accfull[u & 1]);
+                }
+            }
+        }
+        commit_to(drain);  // tensor memory is released only after every MMA has completed
+        if (!mbar_wait(drain, 0u)) failed = true;
+        }
+    }
+    if (failed) atomicOr(&g_f64_error, 1u);
+    __syncwarp();
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    if (warp == 0) {
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(512u) : "memory");
+    }
+}
+
+// U's digits: [unit][K-step][row / 8][K half][row mod 8][8], row = 32 digit + output of the unit
+template <int MODE>
+static void pack(const Op &op, unsigned char *out) {
+    using C = Cfg<MODE>;
+    const double scale = std::ldexp(1.0, 62 - op.f64_su);
+    for (int h = 0; h < C::UNITS; h++)
+        for (int ks = 0; ks < C::KS; ks++) {
+            unsigned short *blk = reinterpret_cast<unsigned short *>(out + (size_t)(h * C::KS + ks) * kBlock);
+            for (int n = 0; n < 32; n++)
+                for (int p = 0; p < 16; p++) {
+                    const int kc = p >> 2, r = p & 3;  // loading lane and its real in the K-step
+                    double u;
+                    if (C::PARTS) {
+                        const int step = MODE == C6 ? ks >> 1 : ks;
+                        const cd z = op.U[(size_t)(32 * h + n) * C::D + kc + 4 * (4 * step + r)];
+                        u = MODE == C6 && (ks & 1) ? z.imag() : z.real();
+                    } else {
+                        const cd z = op.U[(size_t)(16 * h + (n >> 1)) * C::D + kc + 4 * (2 * ks + (r >> 1))];
+                        if (n & 1) u = (r & 1) ? z.real() : z.imag();
+                        else u = (r & 1) ? -z.imag() : z.real();
+                    }
+                    const unsigned long long dg = digit_bytes(u, scale);
+                    for (int j = 0; j < kDigits; j++) {
+                        const int row = 32 * j + n;
+                        blk[(size_t)(row >> 3) * 128 + (p >> 3) * 64 + (row & 7) * 8 + (p & 7)] = half_digit(dg, j);
+                    }
+                }
+        }
+}
+
+static int mode_of(const Op &op) {
+    const int k = (int)op.targets.size();
+    if (k == 6) return op.real_u ? R6 : C6;
+    if (op.real_u) return -1;
+    return k == 5 ? C5 : k == 4 ? C4 : -1;
+}
+
+template <int MODE>
+static void launch(const Args &a, int sms, cudaStream_t st) {
+    using C = Cfg<MODE>;
+    static bool attr = false;
+    if (!attr) {
+        const cudaError_t e =
+            cudaFuncSetAttribute(dense_f64_tc_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+        if (e != cudaSuccess) throw Error(QSIM_ECUDA, std::string("dense_f64_tc_kernel attribute: ") + cudaGetErrorString(e));
+        attr = true;
+    }
+    // one CTA per SM: it holds all 512 tensor-memory columns
+    dense_f64_tc_kernel<MODE><<<(int)std::min<long long>(a.ntiles, sms), kThreads, C::SMEM, st>>>(a);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) throw Error(QSIM_ECUDA, std::string("dense_f64_tc_kernel: ") + cudaGetErrorString(e));
+    note_launches(1, QSIM_KERNEL_DENSE_TC);
+}
+
+#define QSIM_F64TC_SWITCH(m, CALL)  \
+    switch (m) {                    \
+        case C4: CALL(C4); break;   \
+        case C5: CALL(C5); break;   \
+        case R6: CALL(R6); break;   \
+        case C6: CALL(C6); break;   \
+        default: break;             \
+    }
+
+}  // namespace f64tc
+
+// From 2^7 tiles up every SM has one (19 qubits, 4 / 5 / 6 real / 6 targets: 10.7 / 14 / 14 / 20 us here); below, the
+// warp-level kernels spread a state over more SMs (18 qubits: 7.2 / 15 / 14 / 30 us).
+size_t dense_f64_tc_blob_bytes(const Op &op, int n) {
+    using namespace f64tc;
+    size_t bytes = 0;
+    int gb = 0;
+#define QSIM_BYTES(M) bytes = Cfg<M>::BBYTES, gb = Cfg<M>::GB
+    QSIM_F64TC_SWITCH(mode_of(op), QSIM_BYTES)
+#undef QSIM_BYTES
+    return n - (int)(op.targets.size() + op.controls.size()) >= gb + 7 ? bytes : 0;
+}
+
+void dense_f64_tc_pack(const Op &op, unsigned char *out) {
+    using namespace f64tc;
+#define QSIM_PACK(M) pack<M>(op, out)
+    QSIM_F64TC_SWITCH(mode_of(op), QSIM_PACK)
+#undef QSIM_PACK
+}
+
+bool launch_dense_f64_tc(void *state, int n, const Op &op, const void *dig, const void *Ut, int sms, cudaStream_t st) {
+    using namespace f64tc;
+    const int mode = mode_of(op);
+    if (mode < 0) return false;
+    int gb = 0;
+#define QSIM_GB(M) gb = Cfg<M>::GB
+    QSIM_F64TC_SWITCH(mode, QSIM_GB)
+#undef QSIM_GB
+    Args a;
+    std::memset(&a, 0, sizeof(a));
+    unsigned long long used = 0;
+    for (int q : op.targets) used |= 1ull << q;
+    for (int q : op.controls) used |= 1ull << q, a.cmask |= 1ull << q;
+    std::vector<int> fr, fix(op.targets);
+    for (int q = 0; q < n; q++)
+        if (!((used >> q) & 1ull)) fr.push_back(q);
+    if ((int)fr.size() < gb) return false;  // not one tile
+    if ((int)(op.targets.size() + op.controls.size()) + gb > kMaxFix) return false;
+    a.psi = static_cast<double2 *>(state);
+    a.dig = static_cast<const uint4 *>(dig);
+    a.Ut = static_cast<const double2 *>(Ut);
+    a.ntiles = 1ll << ((int)fr.size() - gb);
+    a.diag = op.f64_diag;
+    a.su = op.f64_su;
+    const int k = (int)op.targets.size();
+    for (int v = 0; v < (1 << k); v++)
+        for (int b = 0; b < k; b++)
+            if ((v >> b) & 1) a.amp[v] += 1ll << op.targets[b];
+    for (int b = 0; b < gb; b++) a.grp[b] = 1ll << fr[b];
+    fix.insert(fix.end(), op.controls.begin(), op.controls.end());
+    fix.insert(fix.end(), fr.begin(), fr.begin() + gb);
+    std::sort(fix.begin(), fix.end());
+    a.nfix = (int)fix.size();
+    for (int i = 0; i < a.nfix; i++) a.fix[i] = fix[i];
+#define QSIM_LAUNCH(M) launch<M>(a, sms, st)
+    QSIM_F64TC_SWITCH(mode, QSIM_LAUNCH)
+#undef QSIM_LAUNCH
+    return true;
+}
+
+unsigned dense_f64_read_error() {
+    unsigned v = 0;
+    const cudaError_t e = cudaMemcpyFromSymbol(&v, g_f64_error, sizeof(v));
+    if (e != cudaSuccess) throw Error(QSIM_ECUDA, std::string("reading device status: ") + cudaGetErrorString(e));
+    return v;
+}
+
+void dense_f64_clear_error() {
+    const unsigned z = 0;
+    const cudaError_t e = cudaMemcpyToSymbol(g_f64_error, &z, sizeof(z));
+    if (e != cudaSuccess) throw Error(QSIM_ECUDA, std::string("clearing device status: ") + cudaGetErrorString(e));
+}
+
+}  // namespace qsim

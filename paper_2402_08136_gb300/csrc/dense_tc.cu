@@ -45,6 +45,7 @@
 #include <cstring>
 
 #include "common.h"
+#include "tc_ptx.cuh"
 
 namespace qsim {
 
@@ -55,7 +56,6 @@ namespace tc {
 constexpr int kM = 128;      // groups per tile (MMA M)
 constexpr int kCH = 32;      // K-columns per chunk (16 complex amplitudes)
 constexpr int kMaxFix = 40;
-constexpr unsigned long long kWaitLimitNs = 1000000000ull;  // 1 s
 
 struct Args {
     void *psi;
@@ -72,56 +72,6 @@ struct Args {
     int hi_bit;
 };
 
-__device__ __forceinline__ unsigned smem_u32(const void *p) {
-    return (unsigned)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ uint64_t make_desc(unsigned saddr, unsigned lbo, unsigned sbo) {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr >> 4) & 0x3FFF);
-    d |= (uint64_t)((lbo >> 4) & 0x3FFF) << 16;
-    d |= (uint64_t)((sbo >> 4) & 0x3FFF) << 32;
-    d |= (uint64_t)1 << 46;  // descriptor version for tcgen05
-    return d;                // base offset 0, no swizzle
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t *bar, unsigned count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ unsigned long long global_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %globaltimer;\n" : "=l"(t));
-    return t;
-}
-
-// Bounded wait for the phase with the given parity to complete: gives up after about one
-// second of wall-clock time and returns false.
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity) {
-    const unsigned a = smem_u32(bar);
-    unsigned long long t0 = 0;
-    for (unsigned it = 0;; it++) {
-        unsigned ok;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}\n"
-            : "=r"(ok)
-            : "r"(a), "r"(parity)
-            : "memory");
-        if (ok) return true;
-        if ((it & 255) == 0) {
-            const unsigned long long t = global_ns();
-            if (t0 == 0) t0 = t;
-            else if (t - t0 > kWaitLimitNs) return false;
-        }
-    }
-}
-
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-    asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}\n" ::"r"(smem_u32(bar)) : "memory");
-}
-
 __device__ __forceinline__ void mma_tf32(unsigned d_tmem, uint64_t adesc, uint64_t bdesc, unsigned idesc,
                                          unsigned accumulate) {
     asm volatile(
@@ -131,27 +81,12 @@ __device__ __forceinline__ void mma_tf32(unsigned d_tmem, uint64_t adesc, uint64
         : "memory");
 }
 
-// arrive on `bar` once every tcgen05 operation issued so far by this thread has completed
-__device__ __forceinline__ void commit_to(uint64_t *bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-                     smem_u32(bar))
-                 : "memory");
-}
-
 // TF32 of a finite float, rounded to nearest with ties away from zero: add half a TF32 unit in
 // the last place to the magnitude bits and clear the 13 mantissa bits TF32 drops (integer
 // arithmetic, so the producers' split does not queue on the conversion pipe; same bits as
 // cvt.rna.tf32.f32 for finite inputs, and the state's entries are at most 1 in magnitude)
 __device__ __forceinline__ unsigned to_tf32(float x) {
     return (__float_as_uint(x) + 0x1000u) & 0xFFFFE000u;
-}
-
-__device__ __forceinline__ unsigned long long insert_zeros(unsigned long long x, const int *pos, int cnt) {
-    for (int i = 0; i < cnt; i++) {
-        const int p = pos[i];
-        x = ((x >> p) << (p + 1)) | (x & ((1ull << p) - 1ull));
-    }
-    return x;
 }
 
 template <int K>
@@ -1242,7 +1177,7 @@ unsigned read_device_error() {
     unsigned v = 0;
     cudaError_t e = cudaMemcpyFromSymbol(&v, g_device_error, sizeof(v));
     if (e != cudaSuccess) throw Error(QSIM_ECUDA, std::string("reading device status: ") + cudaGetErrorString(e));
-    return v | dft_tma_read_error() | dft_merge_read_error();  // bit 0 either way: a bounded wait ran out
+    return v | dft_tma_read_error() | dft_merge_read_error() | dense_f64_read_error();  // bit 0 either way: a bounded wait ran out
 }
 
 void clear_device_error() {
@@ -1251,6 +1186,7 @@ void clear_device_error() {
     if (e != cudaSuccess) throw Error(QSIM_ECUDA, std::string("clearing device status: ") + cudaGetErrorString(e));
     dft_tma_clear_error();
     dft_merge_clear_error();
+    dense_f64_clear_error();
 }
 
 }  // namespace qsim

@@ -154,6 +154,7 @@ void dft_fixed_tables(const Op &op, std::vector<int> &out) {
 }
 
 void phase_fixed_table(const std::vector<cd> &v, std::vector<int> &out) {
+    out.reserve(out.size() + 4 * v.size());
     for (const cd &z : v) put(out, std::llrint(z.real() * 0x1p60), std::llrint(z.imag() * 0x1p60));
 }
 }  // namespace qsim

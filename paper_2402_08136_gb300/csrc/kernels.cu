@@ -1148,10 +1148,14 @@ std::vector<unsigned char> pack_device_blob(qsim_circuit *c, int dtype) {
             if (dtype == QSIM_C128) {
                 op.has_f64 = dense_f64_applies(op);
                 if (op.has_f64) {
+                    dense_f64_scale(op);
+                    const size_t tcb = dense_f64_tc_blob_bytes(op, c->n);
+                    op.f64_tc = tcb > 0;
                     align_blob(blob);
                     op.dev_off_tc[slot] = blob.size();
-                    blob.resize(blob.size() + dense_f64_blob_bytes(op));
-                    dense_f64_pack(op, blob.data() + op.dev_off_tc[slot]);
+                    blob.resize(blob.size() + (tcb ? tcb : dense_f64_blob_bytes(op)));
+                    if (tcb) dense_f64_tc_pack(op, blob.data() + op.dev_off_tc[slot]);
+                    else dense_f64_pack(op, blob.data() + op.dev_off_tc[slot]);
                 } else if ((op.sparse_w = sparse_width(op)) > 0) {
                     align_blob(blob);
                     op.dev_off_tc[slot] = blob.size();
@@ -1414,7 +1418,8 @@ void apply_ops(void *state, int n, int dtype, qsim_circuit *c, void *stream, int
                         break;
                 }
                 if (dtype == QSIM_C128 && op.has_f64 &&
-                    launch_dense_f64(state, w, op, base + op.dev_off_tc[slot], dptr, num_sms(), st))
+                    (op.f64_tc ? launch_dense_f64_tc : launch_dense_f64)(state, w, op, base + op.dev_off_tc[slot], dptr,
+                                                                         num_sms(), st))
                     break;
                 if (dtype == QSIM_C128 && op.sparse_w > 0) {
                     launch_sparse(state, w, op, base + op.dev_off_tc[slot], dptr, num_sms(), st);
