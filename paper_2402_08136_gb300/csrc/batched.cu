@@ -25,6 +25,7 @@
 #include <numeric>
 
 #include "common.h"
+#include "dft_fx.cuh"
 
 namespace qsim {
 namespace batch {
@@ -205,6 +206,102 @@ __device__ __forceinline__ V cmulb(V a, V b) {
     return r;
 }
 
+// A twiddle table's entry: complex128 tables hold the integers of the fixed-point passes
+// (dft_fx.cuh), 2^60 (c + i s) in halves.
+__device__ __forceinline__ float2 unit_root(const float2 *t, unsigned i) { return t[i]; }
+__device__ __forceinline__ double2 unit_root(const double2 *t, unsigned i) {
+    const int4 e = reinterpret_cast<const int4 *>(t)[i];
+    const long long c = ((long long)e.x << 32) + e.y, s = ((long long)e.z << 32) + e.w;
+    return make_double2(dftk::fx::to_double(c, -60), dftk::fx::to_double(s, -60));
+}
+
+// complex128 transform stages in 64-bit fixed point, on N amplitudes in shared memory (a CTA's
+// state or a tile of one): in FP64 a stage costs 2 to 4 operations an amplitude, at 2 per clock and SM (a
+// circuit of 13 qubits spent half its time there); integer stages cost their shared-memory traffic.  Every
+// column (the other qubits fixed) gets its own exponent ex[]: 57 bits before the first five stages, and, for
+// wider fields, again before the rest (gr[]: the growth in between).  On return x holds integers, column c in
+// units of 2^(ex[c] - 1079).  False, x as it was, when a column is outside the fixed-point range.
+constexpr int kFxMinK = 5, kFxMaxCols = 256;
+template <int NT>
+__device__ bool fourier_fx(double2 *x, unsigned N, int f0, int K, const int4 *W, bool walsh, int *ex, int tid) {
+    using namespace dftk::fx;
+    const unsigned cols = N >> K, lo = (1u << f0) - 1u;
+    int *gr = ex + kFxMaxCols;
+    auto column = [&](unsigned i) { return (i & lo) | ((i >> (f0 + K)) << f0); };
+    for (unsigned c = tid; c < 2 * kFxMaxCols; c += NT) ex[c] = 0;
+    __syncthreads();
+    bool bad = false;
+    for (unsigned i = tid; i < N; i += NT) {
+        const double2 z = x[i];
+        const unsigned m = max((unsigned)__double2hiint(z.x) & 0x7fffffffu, (unsigned)__double2hiint(z.y) & 0x7fffffffu);
+        const int E = (int)(m >> 20);
+        if (m) {
+            bad |= E > kMaxExp;
+            atomicMax(&ex[column(i)], E);
+        } else {
+            bad |= (__double2loint(z.x) | __double2loint(z.y)) != 0;
+        }
+    }
+    __syncthreads();
+    for (unsigned c = tid; c < cols; c += NT) bad |= ex[c] != 0 && ex[c] < kMinExp;
+    if (__syncthreads_or(bad)) return false;
+    longlong2 *v = reinterpret_cast<longlong2 *>(x);
+    for (unsigned i = tid; i < N; i += NT) {
+        const double2 z = x[i];
+        const int E = ex[column(i)], Es = E ? E : 64;
+        v[i] = make_longlong2(to_fixed<57>(z.x, Es), to_fixed<57>(z.y, Es));
+    }
+    __syncthreads();
+    for (int j = K - 1; j >= 0; j--) {
+        if (j == K - 6) {  // five stages done: back to 57 bits
+            for (unsigned i = tid; i < N; i += NT) {
+                const longlong2 z = v[i];
+                const int hx = (int)(z.x >> 32), hy = (int)(z.y >> 32);
+                const unsigned m = (unsigned)(hx ^ (hx >> 31)) | (unsigned)(hy ^ (hy >> 31));
+                const int g = 7 - __clz((int)m);
+                if (g > 0) atomicMax(&gr[column(i)], g);
+            }
+            __syncthreads();
+            for (unsigned i = tid; i < N; i += NT) {
+                const int g = gr[column(i)];
+                const long long h = (1ll << g) >> 1;
+                const longlong2 z = v[i];
+                v[i] = make_longlong2((z.x + h) >> g, (z.y + h) >> g);
+            }
+            __syncthreads();
+            for (unsigned c = tid; c < cols; c += NT) ex[c] += gr[c];
+        }
+        const int p = f0 + j;
+        const unsigned bit = 1u << p, rmask = (1u << j) - 1u;
+        for (unsigned q = tid; q < N / 2; q += NT) {
+            const unsigned i0 = ((q >> p) << (p + 1)) | (q & (bit - 1u));
+            const longlong2 a = v[i0], b = v[i0 | bit];
+            Z d{a.x - b.x, a.y - b.y};
+            v[i0] = make_longlong2(a.x + b.x, a.y + b.y);
+            if (!walsh) {
+                const unsigned r = (i0 >> f0) & rmask;
+                if (r) d = cmul(d, W[r << (K - 1 - j)]);
+            }
+            v[i0 | bit] = make_longlong2(d.x, d.y);
+        }
+        __syncthreads();
+    }
+    return true;
+}
+// Output i of such a transform (its value sits at v), scaled, times exp(s 2 pi i q / ..) when tw.
+__device__ __forceinline__ double2 fourier_fx_out(longlong2 v, int E, int K, bool tw, unsigned q, const int4 *Tlo,
+                                                  const int4 *Thi, int hT) {
+    using namespace dftk::fx;
+    Z z{v.x, v.y};
+    if (K & 1) {  // 2^(-K/2) = 2^(-floor(K/2)) / sqrt(2)
+        const int4 h = kTwFx.e[4];
+        z = Z{rmul(z.x, h.x, h.y), rmul(z.y, h.x, h.y)};
+    }
+    if (tw) z = cmul(cmul(z, Tlo[q & ((1u << hT) - 1u)]), Thi[q >> hT]);
+    const int e = E - 1022 - 57 - K / 2;
+    return make_double2(to_double(z.x, e), to_double(z.y, e));
+}
+
 // Fourier (DFT) or Walsh-Hadamard transform of the contiguous field f0 .. f0+K-1 inside one
 // circuit: K radix-2 decimation-in-frequency stages (stage j pairs the amplitudes that differ
 // in field bit j; the DFT multiplies the difference by exp(s 2 pi i r / 2^(j+1)), r = the field
@@ -212,7 +309,7 @@ __device__ __forceinline__ V cmulb(V a, V b) {
 // each, then one pass that undoes the digit reversal of the DFT, scales by 2^(-K/2) and
 // applies the output twiddle.  The input twiddle, if any, is a pass of its own first.
 template <typename V, int CS>
-__device__ void op_fourier(V *psi, int n, const BOp &op, const V *data, unsigned vt, bool walsh) {
+__device__ void op_fourier(V *psi, int n, const BOp &op, const V *data, unsigned vt, bool walsh, bool shared, int *ex) {
     constexpr int NT = CS * Threads<V>::n;
     using Rr = decltype(V{}.x);
     const int K = op.k, f0 = op.c0;
@@ -224,8 +321,29 @@ __device__ void op_fourier(V *psi, int n, const BOp &op, const V *data, unsigned
     const unsigned smask = (1u << ns) - 1u, tmask = (1u << hT) - 1u;
     auto tw = [&](unsigned i, unsigned y) -> V {  // exp(s 2 pi i w y / 2^(K+ns))
         const unsigned q = ((i >> s0) & smask) * y;
-        return cmulb(Tlo[q & tmask], Thi[q >> hT]);
+        return cmulb(unit_root(Tlo, q & tmask), unit_root(Thi, q >> hT));
     };
+    if constexpr (sizeof(V) == 16 && CS == 1) {
+        if (shared && K >= kFxMinK && (N >> K) <= kFxMaxCols && twmode != 1) {
+            const int4 *W4 = reinterpret_cast<const int4 *>(W), *lo4 = reinterpret_cast<const int4 *>(Tlo),
+                       *hi4 = reinterpret_cast<const int4 *>(Thi);
+            if (fourier_fx<NT>(psi, N, f0, K, W4, walsh, ex, (int)vt)) {
+                longlong2 *v = reinterpret_cast<longlong2 *>(psi);
+                for (unsigned i = vt; i < N; i += NT) {  // pairs of reversed digits, as below
+                    const unsigned y = (i & fmask) >> f0;
+                    const unsigned yr = walsh ? y : (__brev(y) >> (32 - K));
+                    if (yr < y) continue;
+                    const unsigned ir = (i & ~fmask) | (yr << f0);
+                    const int E = ex[(i & ((1u << f0) - 1u)) | ((i >> (f0 + K)) << f0)];
+                    const longlong2 a = v[i], b = v[ir];
+                    const unsigned w = (i >> s0) & smask;  // the twiddle source lies outside the field
+                    psi[i] = fourier_fx_out(walsh ? a : b, E, K, twmode == 2, w * y, lo4, hi4, hT);
+                    if (ir != i) psi[ir] = fourier_fx_out(a, E, K, twmode == 2, w * yr, lo4, hi4, hT);
+                }
+                return;
+            }
+        }
+    }
     if (twmode == 1) {
         for (unsigned i = vt; i < N; i += NT) psi[i] = cmulb(psi[i], tw(i, (i & fmask) >> f0));
         team_sync<CS>();
@@ -257,7 +375,7 @@ __device__ void op_fourier(V *psi, int n, const BOp &op, const V *data, unsigned
                 psi[i0[e]] = V{a[e].x + b[e].x, a[e].y + b[e].y};
                 if (!walsh) {
                     const unsigned r = (i0[e] >> f0) & rmask;
-                    if (r) d = cmulb(d, W[r << (K - 1 - j)]);
+                    if (r) d = cmulb(d, unit_root(W, r << (K - 1 - j)));
                 }
                 psi[i0[e] | bit] = d;
             }
@@ -290,7 +408,7 @@ __device__ void op_fourier(V *psi, int n, const BOp &op, const V *data, unsigned
 // write per amplitude instead of one per stage.
 template <typename V, int CS>
 __device__ void op_fourier_tiled(V *g, int n, const BOp &op, const V *data, int tid, unsigned rank, bool walsh, V *sm,
-                                 int L) {
+                                 int L, int *ex) {
     constexpr int NT = Threads<V>::n;  // the CTA's threads: a tile belongs to one CTA of the team
     using Rr = decltype(V{}.x);
     const int K = op.k, f0 = op.c0;
@@ -304,7 +422,7 @@ __device__ void op_fourier_tiled(V *g, int n, const BOp &op, const V *data, int 
     const unsigned smask = (1u << ns) - 1u, tmask = (1u << hT) - 1u;
     auto tw = [&](unsigned i, unsigned y) -> V {
         const unsigned q = ((i >> s0) & smask) * y;
-        return cmulb(Tlo[q & tmask], Thi[q >> hT]);
+        return cmulb(unit_root(Tlo, q & tmask), unit_root(Thi, q >> hT));
     };
     auto gidx = [&](unsigned o, unsigned j) -> unsigned {  // tile o, local index j = lane + (y << L)
         const unsigned olo = o & ((1u << mid) - 1u), ohi = o >> mid;
@@ -319,6 +437,20 @@ __device__ void op_fourier_tiled(V *g, int n, const BOp &op, const V *data, int 
             sm[j] = x;
         }
         __syncthreads();
+        if constexpr (sizeof(V) == 16) {
+            if (K >= kFxMinK && (1u << L) <= kFxMaxCols && twmode != 1 &&
+                fourier_fx<NT>(sm, TN, L, K, reinterpret_cast<const int4 *>(W), walsh, ex, tid)) {
+                const longlong2 *v = reinterpret_cast<const longlong2 *>(sm);
+                for (unsigned j = tid; j < TN; j += NT) {
+                    const unsigned y = j >> L, yr = walsh ? y : (__brev(y) >> (32 - K)), gi = gidx(o, j);
+                    g[gi] = fourier_fx_out(v[(j & lmask) | (yr << L)], ex[j & lmask], K, twmode == 2,
+                                           ((gi >> s0) & smask) * y, reinterpret_cast<const int4 *>(Tlo),
+                                           reinterpret_cast<const int4 *>(Thi), hT);
+                }
+                __syncthreads();  // the next tile reuses the buffer
+                continue;
+            }
+        }
         for (int jj = K - 1; jj >= 0; jj--) {
             const int p = L + jj;
             const unsigned bit = 1u << p, rmask = (1u << jj) - 1u;
@@ -331,7 +463,7 @@ __device__ void op_fourier_tiled(V *g, int n, const BOp &op, const V *data, int 
                 sm[i0] = V{a.x + b.x, a.y + b.y};
                 if (!walsh) {
                     const unsigned r = (i0 >> L) & rmask;
-                    if (r) d = cmulb(d, W[r << (K - 1 - jj)]);
+                    if (r) d = cmulb(d, unit_root(W, r << (K - 1 - jj)));
                 }
                 sm[i0 | bit] = d;
             }
@@ -353,7 +485,7 @@ __device__ void op_fourier_tiled(V *g, int n, const BOp &op, const V *data, int 
 
 template <typename R, int CS>
 __device__ void run_op(typename C2<R>::T *psi, int n, const BOp &op, const typename C2<R>::T *data, unsigned vt,
-                       int tid, unsigned rank, typename C2<R>::T *sm, int smem_log) {
+                       int tid, unsigned rank, typename C2<R>::T *sm, int smem_log, int *ex) {
     using V = typename C2<R>::T;
     constexpr int kThreads = CS * Threads<V>::n;  // the team's threads
     const V *d = data + op.data;
@@ -434,6 +566,34 @@ __device__ void run_op(typename C2<R>::T *psi, int n, const BOp &op, const typen
             const unsigned tb = 1u << tq, vmask = (1u << op.nreg) - 1u;
             using Rr = decltype(V{}.x);
             const Rr Cs = d[0].x;
+            // complex128, clock register right below the top qubit: the 2^c0 pairs of a clock value share its
+            // rotation, so each lane of a warp computes that of one of 32 clock values (a division and a square
+            // root in FP64 for every pair took as long as three passes); with a pair per thread or less, each its own
+            if (sizeof(V) == 16 && cnt > (unsigned)kThreads && tq == n - 1 && op.c0 + op.nreg == n - 1) {
+                const unsigned rows = cnt >> op.c0, lane = vt & 31u;
+                for (unsigned b0 = (vt >> 5) * 32u; b0 < rows; b0 += kThreads) {
+                    const unsigned raw = b0 + lane;
+                    const unsigned k = rot ? ((raw >> rot) | ((raw & ((1u << rot) - 1u)) << (op.nreg - rot))) : raw;
+                    Rr sl = 0, cl = 1;
+                    if (k && raw < rows) {
+                        const int ks = (op.k && (k >> (op.nreg - 1))) ? (int)k - (1 << op.nreg) : (int)k;
+                        sl = Cs / (Rr)ks;
+                        if (sl > (Rr)1) sl = (Rr)1;
+                        if (sl < (Rr)-1) sl = (Rr)-1;
+                        const Rr as = sl < 0 ? -sl : sl;
+                        cl = sqrt(((Rr)1 - as) * ((Rr)1 + as));
+                    }
+                    for (unsigned j = 0; j < (1u << op.c0); j++) {
+                        const unsigned e = j * 32u + lane, g = (b0 << op.c0) + e;
+                        const Rr s = __shfl_sync(~0u, sl, (int)(e >> op.c0)), c = __shfl_sync(~0u, cl, (int)(e >> op.c0));
+                        if (g >= cnt) continue;
+                        const V x0 = psi[g], x1 = psi[g | tb];
+                        psi[g] = V{c * x0.x - s * x1.x, c * x0.y - s * x1.y};
+                        psi[g | tb] = V{s * x0.x + c * x1.x, s * x0.y + c * x1.y};
+                    }
+                }
+                break;
+            }
             for (unsigned g = vt; g < cnt; g += kThreads) {
                 const unsigned i0 = ((g >> tq) << (tq + 1)) | (g & (tb - 1u));
                 const unsigned raw = (i0 >> op.c0) & vmask;
@@ -462,8 +622,8 @@ __device__ void run_op(typename C2<R>::T *psi, int n, const BOp &op, const typen
         case B_WALSH: {
             const bool walsh = op.kind == B_WALSH;
             const int L = min((int)op.c0, smem_log - (int)op.k);  // lanes below the field
-            if (psi != sm && L >= 0) op_fourier_tiled<V, CS>(psi, n, op, data, tid, rank, walsh, sm, L);
-            else op_fourier<V, CS>(psi, n, op, data, vt, walsh);
+            if (psi != sm && L >= 0) op_fourier_tiled<V, CS>(psi, n, op, data, tid, rank, walsh, sm, L, ex);
+            else op_fourier<V, CS>(psi, n, op, data, vt, walsh, psi == sm, ex);
             break;
         }
         case B_QPE: {  // data qubits 0..k-1, clock register k..k+nreg-1, split at c0 bits
@@ -541,6 +701,7 @@ __global__ void __launch_bounds__(Threads<typename C2<R>::T>::n) batched_kernel(
     // through two dependent L2 round trips
     unsigned char *stage = smraw + (((size_t)smem_amps * sizeof(V) + 15) & ~(size_t)15);
     __shared__ int cur;
+    __shared__ int ex[sizeof(V) == 16 ? 2 * kFxMaxCols : 1];  // column exponents of the fixed-point passes
     __shared__ double red[3 * (Threads<V>::n >> 5)];
     __shared__ double part[3 * CS];  // team: each CTA's readout sums, gathered in rank 0
     const int tid = threadIdx.x;
@@ -548,6 +709,8 @@ __global__ void __launch_bounds__(Threads<typename C2<R>::T>::n) batched_kernel(
     const unsigned vt = rank * (unsigned)kThreads + (unsigned)tid;
     const int nteams = (int)gridDim.x / CS;
     const int smem_log = 31 - __clz(smem_amps);
+    // the single CTAs' launch may start now, on the SMs that the teams leave free (their circuits are others)
+    if (CS > 1) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     team_sync<CS>();  // a cluster's CTAs have all started before one writes another's shared memory
     for (;;) {
         if (rank == 0 && tid == 0) {
@@ -604,7 +767,7 @@ __global__ void __launch_bounds__(Threads<typename C2<R>::T>::n) batched_kernel(
         }
         team_sync<CS>();
         for (int o = 0; o < c.nops; o++) {
-            run_op<R, CS>(psi, c.n, ops[o], data, vt, tid, rank, sm, smem_log);
+            run_op<R, CS>(psi, c.n, ops[o], data, vt, tid, rank, sm, smem_log, ex);
             team_sync<CS>();
         }
         if (c.flags & 2) {
@@ -655,6 +818,8 @@ __global__ void __launch_bounds__(Threads<typename C2<R>::T>::n) batched_kernel(
             for (unsigned i = tid; i < N; i += kThreads) g[i] = psi[i];
         team_sync<CS>();
     }
+    // ... and ends after the teams' launch, so that what follows on the stream comes after both
+    if (CS == 1) asm volatile("griddepcontrol.wait;\n" ::: "memory");
 }
 
 }  // namespace batch
@@ -832,8 +997,15 @@ bool encode(const Op &op, int dtype, std::vector<unsigned char> &data, BOp &b) {
             b.t[1] = (signed char)(ns == 0 ? 0 : (op.pre ? 1 : 2));
             b.t[2] = (signed char)op.sign;
             b.t[3] = (signed char)((K + ns) / 2);  // the split dft_tables uses
+            b.data2 = (unsigned)(el + W.size());
+            if (dtype == QSIM_C128) {  // the same tables as integers (dft_fx.cuh), 16 bytes an entry too
+                std::vector<int> fixed;
+                dft_fixed_tables(op, fixed);
+                const unsigned char *p = reinterpret_cast<const unsigned char *>(fixed.data());
+                data.insert(data.end(), p, p + fixed.size() * sizeof(int));
+                return true;
+            }
             for (const cd &z : W) put_v(data, dtype, z);
-            b.data2 = (unsigned)(data.size() / vbytes(dtype));
             for (const cd &z : Tlo) put_v(data, dtype, z);
             for (const cd &z : Thi) put_v(data, dtype, z);
             return true;
@@ -1178,9 +1350,22 @@ void launch_batch(qsim_batch *B, cudaStream_t st) {
         note_launches(1, QSIM_KERNEL_BATCHED);
     }
     if (B->count > B->nbig) {
-        batch::batched_kernel<R, 1><<<B->grid, kThreads, B->smem_bytes, st>>>(B->d_circs, B->d_order + B->nbig, B->count - B->nbig,
-                                                                             B->d_counter + 32, B->smem_amps, B->stage_bytes);
-        cudaError_t e = cudaGetLastError();
+        // next to the teams' launch, not after it: the teams of a batch rarely fill the chip, and its single CTAs
+        // need nothing from them (a programmatic dependent launch; see the kernel's griddepcontrol)
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.gridDim = dim3((unsigned)B->grid);
+        cfg.blockDim = dim3(kThreads);
+        cfg.dynamicSmemBytes = B->smem_bytes;
+        cfg.stream = st;
+        cfg.attrs = at;
+        cfg.numAttrs = B->nbig > 0 ? 1 : 0;
+        const batch::BCirc *circs = B->d_circs;
+        const int *order = B->d_order + B->nbig;
+        cudaError_t e = cudaLaunchKernelEx(&cfg, batch::batched_kernel<R, 1>, circs, order, B->count - B->nbig,
+                                           B->d_counter + 32, B->smem_amps, B->stage_bytes);
         if (e != cudaSuccess) throw Error(QSIM_ECUDA, std::string("batched kernel: ") + cudaGetErrorString(e));
         note_launches(1, QSIM_KERNEL_BATCHED);
     }

@@ -135,7 +135,7 @@ __device__ __forceinline__ Z aligned(int4 p, int s) {
     asm("shr.s64 %0, %0, %1;" : "+l"(y) : "r"(s));
     return Z{x, y};
 }
-__device__ __forceinline__ double to_double(long long v, int ex) {  // v 2^(ex - 1023)
+__device__ __forceinline__ double to_double(long long v, int ex) {  // v 2^ex
     const double d = (double)v;
     const int hi = __double2hiint(d);
     return __hiloint2double(hi ? hi + (ex << 20) : 0, __double2loint(d));

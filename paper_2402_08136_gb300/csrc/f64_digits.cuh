@@ -44,7 +44,7 @@ __device__ __forceinline__ void digit_pairs(unsigned long long a, unsigned long 
 
 constexpr float kBiasF = 12582912.0f;  // 1.5 2^23: an FP32 sum started there has its integer in its low bits
 
-// sum_t acc[t] 2^(8 (7 - t)) / 2^SH, rounded to FP64, times 2^(ex - 1023) (0 for a zero sum)
+// sum_t acc[t] 2^(8 (7 - t)) / 2^SH, rounded to FP64, times 2^ex (0 for a zero sum)
 template <bool BIAS, int SH>
 __device__ __forceinline__ double join(const float (&acc)[kDigits], int ex) {
     long long T;
