@@ -725,13 +725,15 @@ __global__ void norm_partials_kernel(const void *state, long long chunk, double 
 // upper half, each half in a fixed order (written by the last pass of a run, or by
 // norm_partials_kernel).
 template <typename R>
-__global__ void norm_final_buf_kernel(const double *buf, const void *state, long long off, int len, double *out);
+__global__ void norm_final_buf_kernel(const double *buf, const void *state, long long off, int len, double *out,
+                                      void *slice = nullptr);
 
 // out[0] = sum of all partials, out[1] = sum of the upper half (ancilla = 1),
-// out[2] = sum over the slice psi[off .. off + len) (ancilla = 1, clock = 0).
+// out[2] = sum over the slice psi[off .. off + len) (ancilla = 1, clock = 0), which is copied to `slice`
+// when that is not NULL.
 template <typename R>
 __device__ void norm_final_body(const double *partials, int nblk, const void *state, long long off, int len,
-                                double *out) {
+                                double *out, void *slice) {
     using V = typename C2<R>::T;
     __shared__ double sh[32];
     double lo = 0.0, hi = 0.0, sl = 0.0;
@@ -742,6 +744,7 @@ __device__ void norm_final_body(const double *partials, int nblk, const void *st
     const V *psi = reinterpret_cast<const V *>(state) + off;
     for (int i = threadIdx.x; i < len; i += blockDim.x) {
         const V z = psi[i];
+        if (slice) reinterpret_cast<V *>(slice)[i] = z;
         const double re = (double)z.x, im = (double)z.y;
         sl = fma(re, re, sl);
         sl = fma(im, im, sl);
@@ -758,13 +761,14 @@ __device__ void norm_final_body(const double *partials, int nblk, const void *st
 
 template <typename R>
 __global__ void norm_final_kernel(const double *partials, int nblk, const void *state, long long off, int len,
-                                  double *out) {
-    norm_final_body<R>(partials, nblk, state, off, len, out);
+                                  double *out, void *slice = nullptr) {
+    norm_final_body<R>(partials, nblk, state, off, len, out, slice);
 }
 
 template <typename R>
-__global__ void norm_final_buf_kernel(const double *buf, const void *state, long long off, int len, double *out) {
-    norm_final_body<R>(buf + 1, (int)buf[0], state, off, len, out);
+__global__ void norm_final_buf_kernel(const double *buf, const void *state, long long off, int len, double *out,
+                                      void *slice) {
+    norm_final_body<R>(buf + 1, (int)buf[0], state, off, len, out, slice);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1514,101 +1518,112 @@ void readout_launch_async(const void *state, int dtype, int n, int nb, cudaStrea
                             cudaMemcpyDeviceToHost, st));
 }
 
+// Device scratch of a readout: from the device's default pool (hhl_readout), or from a pool of the library's own
+// per device (hhl_readout_sums), which keeps up to 64 MiB between calls (it grows by 32 MiB).  The default pool
+// gives its memory back to the driver at every synchronisation, so that a readout, which ends in one, maps memory
+// anew: 169 us of host time against 42 (22 qubits, complex64: 316 -> 191 us per solve).
+namespace {
+class ReadoutScratch {
+  public:
+    ReadoutScratch(size_t bytes, bool own_pool, cudaStream_t st) : st_(st) {
+        if (!own_pool) {
+            const cudaError_t e = cudaMallocAsync(&ptr_, bytes, st);
+            if (e != cudaSuccess) {
+                cudaGetLastError();
+                throw Error(QSIM_ENOMEM, std::string("cudaMallocAsync readout scratch: ") + cudaGetErrorString(e));
+            }
+            return;
+        }
+        static std::mutex mu;
+        static cudaMemPool_t pools[128] = {};
+        int dev = 0;
+        CUDA_OK(cudaGetDevice(&dev));
+        QSIM_REQUIRE(dev >= 0 && dev < 128, "device ordinal out of range");
+        cudaMemPool_t pool;
+        {
+            std::lock_guard<std::mutex> lk(mu);
+            if (pools[dev] == nullptr) {
+                cudaMemPoolProps props;
+                std::memset(&props, 0, sizeof(props));
+                props.allocType = cudaMemAllocationTypePinned;
+                props.location.type = cudaMemLocationTypeDevice;
+                props.location.id = dev;
+                cudaMemPool_t made = nullptr;
+                CUDA_OK(cudaMemPoolCreate(&made, &props));
+                unsigned long long keep = 64ull << 20;
+                CUDA_OK(cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep));
+                pools[dev] = made;
+            }
+            pool = pools[dev];
+        }
+        const cudaError_t e = cudaMallocFromPoolAsync(&ptr_, bytes, pool, st);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            throw Error(QSIM_ENOMEM, std::string("readout scratch: ") + cudaGetErrorString(e));
+        }
+    }
+    ~ReadoutScratch() { cudaFreeAsync(ptr_, st_); }
+    ReadoutScratch(const ReadoutScratch &) = delete;
+    ReadoutScratch &operator=(const ReadoutScratch &) = delete;
+    double *get() const { return static_cast<double *>(ptr_); }
+
+  private:
+    void *ptr_ = nullptr;
+    cudaStream_t st_;
+};
+
+// The sums and the slice, which lies 4 doubles behind them, in one copy (waits for the stream).
+void fetch_readout(const double *out, int dtype, size_t slice_len, cudaStream_t st, double sums[3], cd *slice) {
+    std::vector<unsigned char> host(4 * sizeof(double) + slice_len * 2 * real_size(dtype));
+    CUDA_OK(cudaMemcpyAsync(host.data(), out, host.size(), cudaMemcpyDeviceToHost, st));
+    CUDA_OK(cudaStreamSynchronize(st));
+    std::memcpy(sums, host.data(), 3 * sizeof(double));
+    for (size_t i = 0; i < slice_len; i++) {
+        if (dtype == QSIM_C128) {
+            const double *p = reinterpret_cast<const double *>(host.data()) + 4 + 2 * i;
+            slice[i] = cd(p[0], p[1]);
+        } else {
+            const float *p = reinterpret_cast<const float *>(host.data()) + 8 + 2 * i;
+            slice[i] = cd(p[0], p[1]);
+        }
+    }
+}
+}  // namespace
+
 void readout_device(const void *state, int dtype, int n, int nb, int m, void *stream,
                     double sums[3], cd *slice) {
     (void)m;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const long long N = 1ll << n;
     // fixed block count for a given n: chunks of 2^12 amplitudes, at most 2048 blocks
-    int lg = std::max(1, std::min(11, n - 12));
-    if (n <= 1) lg = 0;
-    const int nblk = 1 << lg;
+    const int nblk = readout_blocks(n);
     const long long chunk = N / nblk;
-    const size_t vb = 2 * real_size(dtype);
     const size_t slice_len = (size_t)1 << nb;
-    void *scratch = nullptr;
-    const size_t scratch_bytes = (size_t)nblk * 8 + 64 + slice_len * vb;
-    cudaError_t e = cudaMallocAsync(&scratch, scratch_bytes, st);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        throw Error(QSIM_ENOMEM, std::string("cudaMallocAsync readout scratch: ") + cudaGetErrorString(e));
-    }
-    double *partials = static_cast<double *>(scratch);
-    double *out = partials + nblk;
+    const ReadoutScratch scratch(((size_t)nblk + 4) * 8 + slice_len * 2 * real_size(dtype), false, st);
+    double *out = scratch.get(), *copy = out + 4, *partials = copy + slice_len * 2 * real_size(dtype) / 8;
     const long long off = N / 2;  // ancilla = 1 (the top qubit), clock = 0
-    try {
-        if (dtype == QSIM_C128) {
-            norm_partials_kernel<double><<<nblk, 256, 0, st>>>(state, chunk, partials);
-            norm_final_kernel<double><<<1, 256, 0, st>>>(partials, nblk, state, off, (int)slice_len, out);
-        } else {
-            norm_partials_kernel<float><<<nblk, 256, 0, st>>>(state, chunk, partials);
-            norm_final_kernel<float><<<1, 256, 0, st>>>(partials, nblk, state, off, (int)slice_len, out);
-        }
-        check_launch("readout kernels", 2, QSIM_KERNEL_READOUT);
-        std::vector<unsigned char> hs(slice_len * vb);
-        double hsum[3];
-        CUDA_OK(cudaMemcpyAsync(hsum, out, 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
-        CUDA_OK(cudaMemcpyAsync(hs.data(), static_cast<const unsigned char *>(state) + off * vb,
-                                slice_len * vb, cudaMemcpyDeviceToHost, st));
-        CUDA_OK(cudaFreeAsync(scratch, st));
-        scratch = nullptr;
-        CUDA_OK(cudaStreamSynchronize(st));
-        for (int i = 0; i < 3; i++) sums[i] = hsum[i];
-        for (size_t i = 0; i < slice_len; i++) {
-            if (dtype == QSIM_C128) {
-                const double *p = reinterpret_cast<const double *>(hs.data()) + 2 * i;
-                slice[i] = cd(p[0], p[1]);
-            } else {
-                const float *p = reinterpret_cast<const float *>(hs.data()) + 2 * i;
-                slice[i] = cd(p[0], p[1]);
-            }
-        }
-    } catch (...) {
-        if (scratch) cudaFreeAsync(scratch, st);
-        throw;
+    if (dtype == QSIM_C128) {
+        norm_partials_kernel<double><<<nblk, 256, 0, st>>>(state, chunk, partials);
+        norm_final_kernel<double><<<1, 256, 0, st>>>(partials, nblk, state, off, (int)slice_len, out, copy);
+    } else {
+        norm_partials_kernel<float><<<nblk, 256, 0, st>>>(state, chunk, partials);
+        norm_final_kernel<float><<<1, 256, 0, st>>>(partials, nblk, state, off, (int)slice_len, out, copy);
     }
+    check_launch("readout kernels", 2, QSIM_KERNEL_READOUT);
+    fetch_readout(out, dtype, slice_len, st, sums, slice);
 }
 
 void readout_device_sums(const void *state, int dtype, int n, int nb, void *stream, const double *buf,
                          double sums[3], cd *slice) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const long long N = 1ll << n;
-    const size_t vb = 2 * real_size(dtype);
     const size_t slice_len = (size_t)1 << nb;
-    const long long off = N / 2;  // ancilla = 1 (the top qubit), clock = 0
-    void *scratch = nullptr;
-    cudaError_t e = cudaMallocAsync(&scratch, 64, st);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        throw Error(QSIM_ENOMEM, std::string("cudaMallocAsync readout scratch: ") + cudaGetErrorString(e));
-    }
-    double *out = static_cast<double *>(scratch);
-    try {
-        if (dtype == QSIM_C128) norm_final_buf_kernel<double><<<1, 256, 0, st>>>(buf, state, off, (int)slice_len, out);
-        else norm_final_buf_kernel<float><<<1, 256, 0, st>>>(buf, state, off, (int)slice_len, out);
-        check_launch("norm_final_buf_kernel", 1, QSIM_KERNEL_READOUT);
-        std::vector<unsigned char> hs(slice_len * vb);
-        double hsum[3];
-        CUDA_OK(cudaMemcpyAsync(hsum, out, 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
-        CUDA_OK(cudaMemcpyAsync(hs.data(), static_cast<const unsigned char *>(state) + off * vb, slice_len * vb,
-                                cudaMemcpyDeviceToHost, st));
-        CUDA_OK(cudaFreeAsync(scratch, st));
-        scratch = nullptr;
-        CUDA_OK(cudaStreamSynchronize(st));
-        for (int k = 0; k < 3; k++) sums[k] = hsum[k];
-        for (size_t k = 0; k < slice_len; k++) {
-            if (dtype == QSIM_C128) {
-                const double *p = reinterpret_cast<const double *>(hs.data()) + 2 * k;
-                slice[k] = cd(p[0], p[1]);
-            } else {
-                const float *p = reinterpret_cast<const float *>(hs.data()) + 2 * k;
-                slice[k] = cd(p[0], p[1]);
-            }
-        }
-    } catch (...) {
-        if (scratch) cudaFreeAsync(scratch, st);
-        throw;
-    }
+    const long long off = 1ll << (n - 1);  // ancilla = 1 (the top qubit), clock = 0
+    const ReadoutScratch scratch(4 * 8 + slice_len * 2 * real_size(dtype), true, st);
+    double *out = scratch.get();
+    if (dtype == QSIM_C128) norm_final_buf_kernel<double><<<1, 256, 0, st>>>(buf, state, off, (int)slice_len, out, out + 4);
+    else norm_final_buf_kernel<float><<<1, 256, 0, st>>>(buf, state, off, (int)slice_len, out, out + 4);
+    check_launch("norm_final_buf_kernel", 1, QSIM_KERNEL_READOUT);
+    fetch_readout(out, dtype, slice_len, st, sums, slice);
 }
 
 // ---------------------------------------------------------------------------------------
