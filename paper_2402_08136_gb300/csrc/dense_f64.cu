@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(Cfg<K, REALU>::THREADS, 1) dense_f64_kernel(co
     constexpr int NT = C::NT, EPL = C::EPL, KS = C::KS;
     extern __shared__ __align__(16) uint4 tabs[];  // [TABS][MT][KS][digit][lane]
     const int tid = threadIdx.x, lane = tid & 31, q = lane & 3, n = lane >> 2;
-    for (int i = tid; i < C::TAB * (C::TABS == 3 ? 2 : 1); i += C::THREADS) {
+    for (int i = tid; i < C::TAB * (C::TABS == 3 ? 2 : 1); i += blockDim.x) {
         uint4 v = a.dig[i];
         tabs[i] = v;
         if (C::TABS == 3 && i >= C::TAB) {  // -Im U
@@ -158,7 +158,8 @@ __global__ void __launch_bounds__(Cfg<K, REALU>::THREADS, 1) dense_f64_kernel(co
         }
     }
     __syncthreads();
-    const long long warps = (long long)gridDim.x * (C::THREADS / 32);
+    const int wpc = blockDim.x / 32;
+    const long long warps = (long long)gridDim.x * wpc;
     // B column n: group (n mod 2) 4 + n / 2 (the store of one accumulator column then covers the
     // lowest group bits), or re / im of group n / 2 for a real U
     const long long in_off = REALU ? a.col[n >> 1] + 8 * (n & 1) : a.col[(n & 1) * 4 + (n >> 1)];
@@ -190,7 +191,7 @@ __global__ void __launch_bounds__(Cfg<K, REALU>::THREADS, 1) dense_f64_kernel(co
                 }
             }
     };
-    long long t = (long long)blockIdx.x * (C::THREADS / 32) + (tid >> 5);
+    long long t = (long long)blockIdx.x * wpc + (tid >> 5);
     if (C::PREFETCH && t < a.ntasks) load(t, x);
     for (; t < a.ntasks; t += warps) {
         if (!C::PREFETCH) load(t, x);
@@ -381,11 +382,16 @@ static void launch(const Args &a, int sms, cudaStream_t st) {
         if (e != cudaSuccess) throw Error(QSIM_ECUDA, std::string("dense_f64_kernel attribute: ") + cudaGetErrorString(e));
         attr = true;
     }
-    const int per_sm = occupancy_cached(reinterpret_cast<const void *>(kern), C::THREADS, C::SMEM);
+    // a state with fewer tasks than the chip has warps is spread over the SMs: full blocks would leave most of them
+    // idle (16 qubits, 4 targets: 512 tasks, 32 blocks of 16 warps 7.0 us, 256 of 2 warps 4.1 us); not where a block
+    // loads 192 KB of digits first (6 targets complex at 17 qubits: 29 us in full blocks, 45 us with one warp each)
+    int wpc = C::THREADS / 32;
+    while (C::SMEM <= 64 * 1024 && wpc > 1 && a.ntasks < (long long)sms * wpc) wpc /= 2;
+    const int threads = wpc * 32;
+    const int per_sm = occupancy_cached(reinterpret_cast<const void *>(kern), threads, C::SMEM);
     QSIM_REQUIRE(per_sm > 0, "dense_f64_kernel does not fit on an SM");
-    const int wpc = C::THREADS / 32;
     const long long grid = std::min<long long>((a.ntasks + wpc - 1) / wpc, (long long)sms * per_sm);
-    kern<<<(int)grid, C::THREADS, C::SMEM, st>>>(a);
+    kern<<<(int)grid, threads, C::SMEM, st>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) throw Error(QSIM_ECUDA, std::string("dense_f64_kernel: ") + cudaGetErrorString(e));
     note_launches(1, QSIM_KERNEL_DENSE_TC);

@@ -143,6 +143,11 @@ bool run_dft(void *state, int n, int dtype, const Op &op, const void *tables, cu
     if (const int v = tune_get(dtype, QSIM_TUNE_DFT_LANES, n))
         L = std::min({v, n - K, (dtype == QSIM_C128 ? 8 : 9) - k1, kMaxLane});
     L = std::max(L, 0);
+    // complex128 fixed-point passes on states of few tiles: narrower tiles down to 32-byte runs, so that more SMs
+    // have one (18 qubits, a 10-qubit field: Walsh 16.1 us with 32 tiles, 11 with 128, transform 22.7 and 14.5; the
+    // state is in L2, where 32-byte runs cost little)
+    if (dtype == QSIM_C128 && contig && K >= 5 && tune_get(dtype, QSIM_TUNE_DFT_LANES, n) == 0)
+        while (L > std::max(1, 6 - k1) && n - K - L < 7) L--;
     unsigned long long fmask = 0;
     for (int q : op.targets) fmask |= 1ull << q;
     std::vector<int> fix(op.targets.begin(), op.targets.end());

@@ -1613,9 +1613,28 @@ void readout_device(const void *state, int dtype, int n, int nb, int m, void *st
     fetch_readout(out, dtype, slice_len, st, sums, slice);
 }
 
+// A readout on a stream of its own comes after what is already enqueued on the device's default stream, where the
+// run it reads may have been replayed (allocating from the default pool used to take long enough for that).
+static void after_default_stream(cudaStream_t st) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (st == nullptr || st == cudaStreamLegacy) return;
+    // a blocking stream under capture forbids touching the default stream (the query does not disturb it)
+    if (cudaStreamIsCapturing(cudaStreamLegacy, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return;
+    }
+    cudaEvent_t ev = nullptr;
+    CUDA_OK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+    cudaError_t e = cudaEventRecord(ev, cudaStreamLegacy);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ev, 0);
+    cudaEventDestroy(ev);
+    CUDA_OK(e);
+}
+
 void readout_device_sums(const void *state, int dtype, int n, int nb, void *stream, const double *buf,
                          double sums[3], cd *slice) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    after_default_stream(st);
     const size_t slice_len = (size_t)1 << nb;
     const long long off = 1ll << (n - 1);  // ancilla = 1 (the top qubit), clock = 0
     const ReadoutScratch scratch(4 * 8 + slice_len * 2 * real_size(dtype), true, st);
