@@ -25,7 +25,7 @@
 // are output amplitudes, written back in place.  U's digits sit in shared memory in fragment order.
 // Group bits are the lowest free qubits, so a warp's load covers whole 128-byte lines.
 //
-// Not all gates take this form (dense_f64_applies): one whose rows are mostly zeros keeps the FP64
+// Not all gates take this form (dense_f64_applies): those with mostly zero rows keep the FP64
 // kernels, which are exact on permutations; rows that only scale their own amplitude (the padding of
 // an eigenvector matrix, a controlled gate written as a dense one) are computed in FP64 on the way out.
 // A tile with a group that is not finite, or whose largest exponent is far from 1, is computed in
@@ -424,16 +424,21 @@ static unsigned long long diagonal_rows(const Op &op) {
     return diag;
 }
 
-// Gates of 1..6 targets whose rows are mostly nonzero.  A sum of a few terms that misses the group's
-// largest value is more exact in FP64 than relative to that value (a permutation is exact), so a
-// gate with a row of at most half its entries nonzero (diagonal rows and columns apart) stays in FP64.
+// Gates of 1..6 targets with mostly nonzero rows.  A sum of a few terms that misses the group's largest value
+// is more exact in FP64 than relative to that value (a permutation is exact), so a gate with a row of at most half
+// its entries nonzero (diagonal rows and columns apart) stays in FP64 where the row form makes that cheap
+// (sparse_width).  A gate that mixes such rows with full ones, a quarter of its entries nonzero at least, comes here
+// all the same: the plain kernel would multiply all of its zeros (the eigenvectors of a grid that falls apart
+// without its slack bus, 64 x 64 in blocks of 63 and 1: 30.8 ms in FP64 on 2^27 amplitudes, 1.5 ms here).  The error
+// of its short rows is then 2^-57 of the group's largest value, as that of the full ones.
 bool dense_f64_applies(const Op &op) {
     const int k = (int)op.targets.size();
     if (op.kind != OP_DENSE || k < 1 || k > 6) return false;
     const int D = 1 << k;
     const unsigned long long diag = diagonal_rows(op);
     double top = 0.0;
-    int live = 0;
+    int live = 0, all = 0;
+    bool short_rows = false;
     for (int r = 0; r < D; r++) live += !((diag >> r) & 1ull);
     for (int r = 0; r < D; r++) {
         if ((diag >> r) & 1ull) continue;
@@ -443,8 +448,10 @@ bool dense_f64_applies(const Op &op) {
             top = std::max(top, std::max(std::fabs(u.real()), std::fabs(u.imag())));
             if (!((diag >> c) & 1ull)) nz += u != cd(0.0, 0.0);
         }
-        if (2 * nz <= live) return false;
+        short_rows = short_rows || 2 * nz <= live;
+        all += nz;
     }
+    if (short_rows && (sparse_width(op) > 0 || 4 * all < live * live)) return false;
     return live > 0 && top > std::ldexp(1.0, -100) && top < std::ldexp(1.0, 100);
 }
 

@@ -103,3 +103,25 @@ def test_few_groups(qs, k, dtype, eps):
             out, ref = apply(qs, psi, n, t, U, ctl, dtype), oracle(psi, t, U, ctl)
             # a sum of 2^(k+1) products, rounded after each, on both sides
             assert np.max(np.abs(out - ref)) <= 2 * (2.0 ** (k + 1) + 2) * eps * 2.0 ** (k / 2) * np.max(np.abs(psi))
+
+
+@pytest.mark.parametrize("k,blocks,real", [(4, (13, 3), False), (5, (31, 1), True), (6, (63, 1), True), (6, (40, 24), True),
+                                           (6, (50, 13, 1), False)])
+def test_blocks_of_different_size(qs, k, blocks, real):
+    """Short rows next to full ones (a grid that falls apart): on the digit kernels, within their bound."""
+    rng = np.random.default_rng(k)
+    D = 1 << k
+    U = np.zeros((D, D), dtype=np.complex128)
+    at = 0
+    for b in blocks:
+        Z = rng.standard_normal((b, b)) + (0 if real else 1j * rng.standard_normal((b, b)))
+        U[at:at + b, at:at + b] = np.linalg.qr(Z)[0]
+        at += b
+    U = U[rng.permutation(D)][:, rng.permutation(D)]
+    for n in (k + 6, k + 14):
+        t = synth.random_targets(rng, n, k)
+        psi = synth.gaussian_state_np(k, n)
+        before = qs.qsim_launch_counts()["dense_tc"]
+        out = apply(qs, psi, n, t, U)
+        assert qs.qsim_launch_counts()["dense_tc"] > before
+        assert np.max(np.abs(out - oracle(psi, t, U))) <= (2.0 * D + 2) * 2.0 ** -53 * 2.0 ** (k / 2) * np.max(np.abs(psi))
