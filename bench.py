@@ -292,6 +292,8 @@ def run_gates(args, ws, rank, dtype_name):
 
     # which kernel the library launches for each gate (its per-family launch counters)
     fam_of = [launched_family(qs, lambda c=c: qs.qsim_apply(st, c, stream)) for c in circs]
+    if dtype_name == "c128":  # the tensor-core family's digit kernels
+        fam_of = [f.replace(FAMILY_KERNEL["dense_tc"], "dense_f64_kernel+dense_f64_tc_kernel") for f in fam_of]
     for _ in range(args.warmup):
         step()
     torch.cuda.synchronize()
@@ -341,23 +343,11 @@ def run_gates(args, ws, rank, dtype_name):
     traffic = None
     if tr is not None:
         traffic = round(tr["bytes_per_amp"] * (1 << n))
-    if dtype_name == "c64":
-        roofline = {"bound": "hbm", "kernel": dom, "achieved": achieved, "peak": hbm,
-                    "peak_kind": peak_kind + " copy bandwidth (MEASURED_PEAKS.json hbm_gbs)",
-                    "unit": "GB/s", "frac": round(achieved / hbm, 4), "traffic": traffic,
-                    "traffic_source": tr["source"] if tr else None,
-                    "bytes_per_launch": bytes_per_gate}
-    else:
-        # complex128: FP64 FMA bound (a dense k-qubit gate is 8 * 2^k real flops per amplitude)
-        sel = [i for i, k in enumerate(ks) if fam_of[i] == dom]
-        fl = sum(8.0 * (2 ** ks[i]) * (1 << n) for i in sel) * args.steps
-        tf = fl / (fams[dom]["ms_total"] / 1e3) / 1e12
-        roofline = {"bound": "alu", "kernel": dom, "achieved": round(tf, 4),
-                    "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                    "peak_kind": "nominal GB300 FP64 rate (1.25 TFLOP/s; a probe measured 1.21)",
-                    "frac": round(tf / FP64_PEAK_TFLOPS, 4), "traffic": traffic,
-                    "traffic_source": tr["source"] if tr else None,
-                    "hbm_achieved_gbs": achieved}
+    roofline = {"bound": "hbm", "kernel": dom, "achieved": achieved, "peak": hbm,
+                "peak_kind": peak_kind + " copy bandwidth (MEASURED_PEAKS.json hbm_gbs)",
+                "unit": "GB/s", "frac": round(achieved / hbm, 4), "traffic": traffic,
+                "traffic_source": tr["source"] if tr else None,
+                "bytes_per_launch": bytes_per_gate}
 
     # end to end through the public API from pinned host memory
     host_in = synth.gaussian_state_torch(seed, n, dtype, "cpu", chunk=1 << 22, normalize=True) \
@@ -549,7 +539,8 @@ def fourier_pass_roofline(qs, torch, launches: int = 10):
 
 def sub_hhl27(args, ws, rank):
     """The 27-qubit precision-form solve: complex64 (structured phase estimation, QFTs as
-    passes, fused dense gates on the tensor cores) and complex128 (FP64 SIMT), both through
+    passes, fused dense gates on the tensor cores) and complex128 (digit products and fixed-point
+    passes), both through
     hhl_run + hhl_readout; solves/s, latency, readout error against the classical A^-1 b; the
     Fourier-pass kernel's roofline; the final states kept on the host for the comparison with
     the full-size oracle (oracle_hhl27_compare, run after every GPU measurement)."""

@@ -46,7 +46,7 @@ extern "C" {
 
 /* ---- state dtypes ---------------------------------------------------------------------- */
 #define QSIM_C64 1  /* complex64: FP32 state; gate arithmetic FP32 (dense k>=4 on tensor cores) */
-#define QSIM_C128 2 /* complex128: FP64 state and FP64 gate arithmetic                          */
+#define QSIM_C128 2 /* complex128: FP64 state; gate arithmetic exact to FP64 rounding or better   */
 
 typedef struct qsim_circuit qsim_circuit; /* gate list (unfused or fused)                       */
 typedef struct hhl_circuit hhl_circuit;   /* HHL problem + its unfused gate list                */
@@ -182,8 +182,8 @@ unsigned long long qsim_launch_count(void);
 
 /* The same count split by kernel family (so a caller can tell which kernel ran an operation):
  * counts[i] for family i (QSIM_KERNEL_*), i < n; entries beyond the families are 0. */
-#define QSIM_KERNEL_DENSE_SIMT 0   /* dense gates, SIMT (dense_pipe_kernel, dense_tile_kernel)      */
-#define QSIM_KERNEL_DENSE_TC 1     /* dense gates on the tensor cores (complex64)                   */
+#define QSIM_KERNEL_DENSE_SIMT 0   /* dense gates, SIMT (tiled, mostly-zero rows, few groups)       */
+#define QSIM_KERNEL_DENSE_TC 1     /* dense gates on the tensor cores                               */
 #define QSIM_KERNEL_FOURIER 2      /* Fourier / Walsh-Hadamard passes, thread loads                 */
 #define QSIM_KERNEL_FOURIER_TMA 3  /* Fourier / Walsh-Hadamard passes, bulk-copy (TMA) tiles       */
 #define QSIM_KERNEL_EXPAND 4       /* write-only broadcast of a pass on an unwritten field          */
@@ -400,7 +400,10 @@ int hhl_readout(const void *state, int dtype, const hhl_circuit *h, void *stream
  * controls in the transposed 6-target or the real 7-target form (the eigenvector rotation V that
  * ends the structured HHL circuit), else by a reduction pass after it.  Device-only, so it can be captured into a CUDA graph.  hhl_readout_sums is
  * hhl_readout taking those partials instead of reducing the state again; the state must not
- * have changed since the hhl_run_sums that wrote sums_device.  Errors: EINVAL, ENOMEM, ECUDA. */
+ * have changed since the hhl_run_sums that wrote sums_device.  Its device scratch comes from a
+ * memory pool of the library's own (up to 64 MiB kept per device until the process ends); on a
+ * stream of its own it also waits for work already enqueued on the default stream.
+ * Errors: EINVAL, ENOMEM, ECUDA. */
 #define QSIM_READOUT_SUMS_DOUBLES 4096
 int hhl_run_sums(void *state, int dtype, const hhl_circuit *h, const qsim_circuit *c, void *stream,
                  double *sums_device);
@@ -433,9 +436,10 @@ int hhl_batch_create(const hhl_circuit *const *hs, const qsim_circuit *const *fu
  * copy, no synchronization; each kernel resets its own work counter when it ends), so the call
  * can be captured into a CUDA graph.  Runs of one batch must not overlap (same stream, or
  * ordered).  Circuits whose state exceeds 2^13 (complex128) or 2^14 (complex64) amplitudes
- * run first, each on a team of 4 CTAs (a thread-block cluster) that splits every operation
- * and updates the state in place; then every other circuit runs on one CTA with its state in
- * shared memory.  Within each launch circuits go most expensive first.  A circuit always runs
+ * run each on a team of 4 CTAs (a thread-block cluster) that splits every operation
+ * and updates the state in place; every other circuit runs on one CTA with its state in
+ * shared memory, in a second launch that starts on the SMs the teams leave free and ends after
+ * them.  Within each launch circuits go most expensive first.  A circuit always runs
  * on the same kind of team in a fixed order, so its result is bit-identical whatever else is
  * in the batch; it equals qsim_apply of the same circuit up to rounding (different kernels).
  * Errors: EINVAL, ECUDA. */

@@ -93,8 +93,9 @@ struct Op {
     int pre = 0;                // OP_DFT
     // device offsets (bytes) into the circuit's device blob, per dtype
     size_t dev_off[2] = {0, 0};
-    // second table, per dtype: complex64 dense ops with 4..7 targets, the TF32 hi/lo split of
-    // the real form (tensor cores); OP_QPE_PHASE, the high half of its two-table split
+    // second table, per dtype: complex64 dense ops with 3..7 targets, the TF32 hi/lo split of
+    // the real form (tensor cores); complex128 dense ops, U's digits or its nonzero entries;
+    // OP_QPE_PHASE, the high half of its two-table split
     size_t dev_off_tc[2] = {0, 0};
     bool has_tc = false;
     // complex64 dense op of 1..5 targets on qubit 0 or 1 widened with identity qubits to the

@@ -30,6 +30,11 @@
 // an eigenvector matrix, a controlled gate written as a dense one) are computed in FP64 on the way out.
 // A tile with a group that is not finite, or whose largest exponent is far from 1, is computed in
 // the plain FP64 form by the same warp (plain_tile).
+//
+// 26 qubits, FP64 form -> this one, TB/s: k = 1 2.26 -> 3.83, 2 1.17 -> 3.8, 3 0.62 -> 3.8, 4 0.31 -> 2.45, 5 0.16 -> 1.35,
+// 6 0.072 -> 0.76 (from 4 targets on, large states take dense_f64_tc.cu).  k <= 3 is bound by issue slots (splitting and
+// joining the digits), wider gates by the MMAs.  Error against long double 4.6e-17 of the largest amplitude
+// (FP64 form 7e-17 to 3.5e-16).
 #include <cuda_runtime.h>
 #include <cuda_fp16.h>
 

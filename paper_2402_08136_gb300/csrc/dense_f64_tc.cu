@@ -23,6 +23,13 @@
 // 4 amplitudes of 8 groups (the lowest targets and free qubits: whole lines).  Roles meet at mbarriers only,
 // every wait is bounded, tensor memory is freed after the last MMA has completed (as in dense_tc.cu).
 // A tile with a group outside the fixed-point range is computed in FP64 by the reading warps (plain_tile).
+//
+// 26 qubits, dense_f64.cu's form -> this one, TB/s: 4 targets 2.42 -> 3.54, 5 1.40 -> 2.9, 6 0.77 -> 1.63, 6 with a real U
+// 1.57 -> 2.8.  What bounds it: issue slots for splitting and joining the digits (0.59 instructions a clock and
+// scheduler at 4 targets, 0.50 at 5; the tensor pipe at 21 to 39 %); at 6 complex targets the MMAs and the joining take turns, as tensor
+// memory holds one tile's two units and no more.  The FP64 pipe is at 17 to 37 %: its last
+// conversion only, scaled rows apart, whose products sit behind a branch of their own (as predicated instructions
+// they passed the pipe for every row: 69 % of it).
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -14,6 +14,11 @@
 // An error of a few units of 2^-56 of a column's largest value is left, below the FP64 form's.
 // Tile, layout and thread mapping are dft_kernel's (see dft_impl.cuh).  A tile with a point that is
 // not finite, or a thread's largest exponent far from 1, is transformed in FP64 (plain_tile).
+//
+// 10 qubits of a 25-qubit state, FP64 form -> this one: Walsh-Hadamard 2030 -> 350 us, Fourier 2800 -> 515 us, Fourier with
+// twiddles 2823 -> 620 us (1 GiB moved: 160 us at the copy rate).  What bounds it: issue slots (integer multiply-adds and
+// shifts).  9 and 10 qubits run in three steps of 16 x 8 x (4 or 8) points: two steps of 32 points took 1044 us, their
+// code outgrew the instruction cache.
 #pragma once
 #include "dft_impl.cuh"
 
