@@ -365,7 +365,9 @@ __global__ void __launch_bounds__(256, 1) dft_fx_kernel(const __grid_constant__ 
 // step 1 transforms over v (output digit a), step 2 over the high part of u = u2 + N3 v2 (digit a2),
 // step 3 over u2 (digit b2); y' = a + 16 (a2 + 8 b2).  The tile's element (a, u) sits in row a Nr + u.
 // The points are aligned to the column's exponent when step 2 reads them.
-template <int K, int SGN, int KIND>
+// TILE (see tile_twiddles): the products of the two twiddle tables' entries are made once a tile, 2^K of them for
+// 2^(K + L) points, while step 1's loads are in flight.
+template <int K, int SGN, int KIND, bool TILE>
 __global__ void __launch_bounds__(512, 1) dft_fx3_kernel(const __grid_constant__ DftArgs a) {
     constexpr bool WALSH = KIND == 1, INV = KIND == 2;
     constexpr int RA = 16, RB = 8, RC = 1 << (K - 7), NR = RB * RC, KN = 1 << K;
@@ -374,7 +376,8 @@ __global__ void __launch_bounds__(512, 1) dft_fx3_kernel(const __grid_constant__
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int4 *S = reinterpret_cast<int4 *>(smem_raw);
     int4 *Ws = S + (KN << L);
-    int4 *Ts = Ws + (WALSH ? 0 : KN);
+    int4 *TW = Ws + (WALSH ? 0 : KN);
+    int4 *Ts = TW + (TILE ? KN : 0);
     const int ntlo = 1 << a.hT, nthi = 1 << (K + a.ns - a.hT);
     double2 *cs = reinterpret_cast<double2 *>(Ts + (a.tw_smem ? ntlo + nthi : 0));
     int *ex = reinterpret_cast<int *>(cs + (INV && a.inv_shared ? KN : 0));  // [u][lane]
@@ -417,6 +420,14 @@ __global__ void __launch_bounds__(512, 1) dft_fx3_kernel(const __grid_constant__
             const long long step = (long long)NR << a.f0;
 #pragma unroll
             for (int v = 0; v < RA; v++) x[v] = src[v * step];
+            if (TILE)  // w is the tile's: its twiddles once, not once a lane
+#pragma unroll 1
+                for (int i = tid; i < KN; i += nthr) {
+                    const unsigned q = w * (unsigned)i;
+                    const int4 t = Tlo[q & tmask];
+                    const Z y = cmul(Z{((long long)t.x << 32) + t.y, ((long long)t.z << 32) + t.w}, Thi[q >> a.hT]);
+                    TW[i] = make_int4(high(y.x), low(y.x), high(y.y), low(y.y));
+                }
             unsigned m = 0, lows = 0;
 #pragma unroll
             for (int v = 0; v < RA; v++) {
@@ -505,7 +516,9 @@ __global__ void __launch_bounds__(512, 1) dft_fx3_kernel(const __grid_constant__
                     const int4 h = kTwFx.e[4];
                     v = Z{rmul(v.x, h.x, h.y), rmul(v.y, h.x, h.y)};
                 }
-                if (!WALSH && a.twmode == 2) {
+                if (TILE) {
+                    v = cmul(v, TW[y]);
+                } else if (!WALSH && a.twmode == 2) {
                     const unsigned q = w * (unsigned)y;
                     v = cmul(cmul(v, Tlo[q & tmask]), Thi[q >> a.hT]);
                 }
@@ -528,18 +541,21 @@ __global__ void __launch_bounds__(512, 1) dft_fx3_kernel(const __grid_constant__
     }
 }
 
-template <int K, int SGN, int KIND>
+template <int K, int SGN, int KIND, bool TILE = false>
 void launch(DftArgs a, cudaStream_t st) {
     constexpr bool THREE = K >= 9;
     const size_t KN = (size_t)1 << K, N1 = THREE ? KN / 16 : (size_t)1 << (K / 2), NL = (size_t)1 << a.L;
     const int threads = (int)(N1 * NL);
     size_t smem = 16 * ((KN << a.L) + (THREE ? 0 : N1 * NL) + (KIND == 1 ? 0 : KN)) + 4 * (N1 * NL + 2 * NL);
     if (KIND == 2 && a.inv_shared) smem += 16 * KN;
+    if (TILE) smem += 16 * KN;
     const size_t tw = 16 * (((size_t)1 << a.hT) + ((size_t)1 << (K + a.ns - a.hT)));
-    a.tw_smem = a.ns > 0 && smem + tw <= 220 * 1024 ? 1 : 0;  // read once per amplitude
+    // the tables too, unless they would take a second CTA's room (read once per amplitude, or once a tile)
+    a.tw_smem = a.ns > 0 && smem + tw <= (TILE && threads <= 256 ? 112 : 220) * 1024 ? 1 : 0;
     if (a.tw_smem) smem += tw;
     void (*kern)(const DftArgs) = nullptr;
-    if constexpr (THREE) kern = dft_fx3_kernel<K, SGN, KIND>;
+    if constexpr (TILE) kern = dft_fx3_kernel<K, SGN, KIND, TILE>;
+    else if constexpr (THREE) kern = dft_fx3_kernel<K, SGN, KIND, false>;
     else kern = dft_fx_kernel<K, SGN, KIND>;
     static bool attr = false;
     if (!attr) {
@@ -555,8 +571,26 @@ void launch(DftArgs a, cudaStream_t st) {
     note_launches(1, QSIM_KERNEL_FOURIER);
 }
 
+// Twiddles as one table a tile (no lane qubit is a twiddle source): a point then shares the product of the two
+// tables' entries with the other lanes.  25 qubits, 10-qubit field, 8 lanes: 637 -> 569 us; 4 lanes 830 -> 713 us (tables
+// left in global memory, so that two CTAs fit); with 2 lanes half of the products are left and the table's
+// traffic comes on top.  Forms of their own: as a branch of the one kernel they cost the passes without a table 2 %.
+inline bool tile_twiddles(const DftArgs &a) {
+    bool ok = a.twmode == 2 && a.ns > 0 && a.L >= 2;
+    for (int i = 0; i < a.ns; i++)
+        for (int j = 0; j < a.L; j++) ok = ok && a.spos[i] != a.lpos[j];
+    return ok;
+}
+
 template <int K>
 void launch_k(const DftArgs &a, int sign, int kind, cudaStream_t st) {
+    if constexpr (K >= 9)
+        if (kind != 1 && tile_twiddles(a)) {
+            if (kind == 2) launch<K, -1, 2, true>(a, st);
+            else if (sign > 0) launch<K, 1, 0, true>(a, st);
+            else launch<K, -1, 0, true>(a, st);
+            return;
+        }
     if (kind == 2) launch<K, -1, 2>(a, st);
     else if (kind == 1) launch<K, 1, 1>(a, st);
     else if (sign > 0) launch<K, 1, 0>(a, st);

@@ -73,6 +73,18 @@ def test_fields(qs, K, kind):
         assert np.max(np.abs(out - ref)) <= 8 * (K + 2) * 2.0 ** -53 * 2.0 ** (K / 2) * np.max(np.abs(psi)), (n, f0, s)
 
 
+@pytest.mark.parametrize("kind", ["dft+", "dft-"])
+@pytest.mark.parametrize("K", [9, 10])
+def test_tile_twiddles(qs, K, kind):
+    """Sources on both sides of the rule for one twiddle table a tile: none, one or all of them in a lane; tiles of
+    few and of many lanes; more tiles than SMs."""
+    for n, f0, src in ((K + 8, 4, [K + 4, K + 5]), (K + 9, 4, [3]), (K + 9, 5, [4, K + 5, K + 8]), (K + 9, 3, [2, K + 4]),
+                       (K + 11, 4, [0, 1, 2, 3]), (K + 11, 4, [K + 4 + i for i in range(7)])):
+        psi = synth.gaussian_state_np(K + f0, n)
+        out, ref = run(qs, psi, n, f0, K, kind, src), reference(psi, n, f0, K, kind, src)
+        assert np.max(np.abs(out - ref)) <= 8 * (K + 2) * 2.0 ** -53 * 2.0 ** (K / 2) * np.max(np.abs(psi)), (n, f0, src)
+
+
 @pytest.mark.parametrize("kind", ["walsh", "dft+", "dft-"])
 @pytest.mark.parametrize("K", [6, 9, 10])
 def test_values(qs, K, kind):
