@@ -56,6 +56,11 @@ constexpr int kThreads = (kMmaWarp + 4) * 32;  // the issuing warp's group of fo
 constexpr int kProdRegs = 128, kEpiRegs = 80, kMmaRegs = 56;
 constexpr int kSlot = kDigits * 4096;  // one K-step of a tile: 8 digits x 128 rows x 16 FP16
 constexpr int kBlock = 8192;           // U's digits of one unit and K-step: 256 rows x 16 FP16
+// Slots of what the loading warps tell the reading ones about a tile (exponents, odd marks).  Tile t is written once
+// its first K-step has a ring slot, so the MMAs of the K-step SLOTS before it are complete, and they had waited for
+// the unit two before theirs to be read: tile t - 4 with 4 targets (2 tiles in the ring, 2 in tensor memory), tile
+// t - 2 in the other modes.  Every earlier tile has been read when slot t mod 4 is written.
+constexpr int kTiles = 4;
 
 enum Mode { C4 = 0, C5 = 1, R6 = 2, C6 = 3 };
 
@@ -75,7 +80,7 @@ struct Cfg {
     static constexpr int SH = RED > 64 ? 13 : 12;
     static constexpr int BBYTES = UNITS * KS * kBlock;
     static constexpr int STAGE = kEpiWarps * 2048;
-    static constexpr int SMEM = BBYTES + SLOTS * kSlot + STAGE + 4 * 128 * 4 + 16 + 8 * (2 * SLOTS + 5) + 16;
+    static constexpr int SMEM = BBYTES + SLOTS * kSlot + STAGE + kTiles * (128 * 4 + 8) + 8 * (2 * SLOTS + 5) + 16;
 };
 
 struct Args {
@@ -186,15 +191,14 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
     extern __shared__ __align__(1024) unsigned char sm[];
     unsigned char *ring = sm + C::BBYTES;
     unsigned char *stage = ring + SLOTS * kSlot;
-    int *exps = reinterpret_cast<int *>(stage + C::STAGE);  // [4 tiles][128 rows]
-    int *odd = exps + 4 * 128;                              // [4 tiles]: the tile takes plain_tile
-    uint64_t *full = reinterpret_cast<uint64_t *>(odd + 4);
+    int *exps = reinterpret_cast<int *>(stage + C::STAGE);  // [kTiles][128 rows]
+    uint64_t *odd = reinterpret_cast<uint64_t *>(exps + kTiles * 128);  // [kTiles], a byte per loading warp: plain_tile if any is set
+    uint64_t *full = odd + kTiles;
     uint64_t *empty = full + SLOTS, *accfull = empty + SLOTS, *accempty = accfull + 2, *drain = accempty + 2;
     unsigned *tslot = reinterpret_cast<unsigned *>(drain + 1);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     for (int i = tid; i < C::BBYTES / 16; i += kThreads) reinterpret_cast<uint4 *>(sm)[i] = a.dig[i];
-    if (tid < 4) odd[tid] = 0;
     if (tid == 0) {
         for (int i = 0; i < SLOTS; i++) {
             mbar_init(&full[i], kProdWarps);
@@ -248,6 +252,7 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
         const unsigned col = (unsigned)((kc >> 1) * 128 + (kc & 1) * 8);
         for (long long t = 0; t < ntl && !failed; t++) {
             int Er[ITEMS], Ei[ITEMS];
+            bool out = false;  // a group is outside the fixed-point range
 #pragma unroll
             for (int it = 0; it < ITEMS; it++) {
                 unsigned mr = 0, mi = 0, low = 0;
@@ -273,17 +278,24 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
                         if (!mag_bits(x[it][e].x)) low |= (unsigned)__double2loint(x[it][e].x);
                         if (!mag_bits(x[it][e].y)) low |= (unsigned)__double2loint(x[it][e].y);
                     }
-                if (Er[it] < kMinExp || Er[it] > kMaxExp || Ei[it] < kMinExp || Ei[it] > kMaxExp || low) odd[t & 3] = 1;
+                out |= Er[it] < kMinExp || Er[it] > kMaxExp || Ei[it] < kMinExp || Ei[it] > kMaxExp || low;
+            }
+            out = __any_sync(~0u, out);
+            auto post = [&] {  // after the wait for the tile's first ring slot (see kTiles)
+                int *ex = exps + (t % kTiles) * 128;
                 if (kc == 0) {
-                    int *ex = exps + (t & 3) * 128;
-                    if (PARTS) {
-                        ex[2 * (8 * warp + r8)] = Er[it];
-                        ex[2 * (8 * warp + r8) + 1] = Ei[it];
-                    } else {
-                        ex[64 * it + 8 * warp + r8] = Er[it];
+#pragma unroll
+                    for (int it = 0; it < ITEMS; it++) {
+                        if (PARTS) {
+                            ex[2 * (8 * warp + r8)] = Er[it];
+                            ex[2 * (8 * warp + r8) + 1] = Ei[it];
+                        } else {
+                            ex[64 * it + 8 * warp + r8] = Er[it];
+                        }
                     }
                 }
-            }
+                if (lane == 0) reinterpret_cast<unsigned char *>(odd + t % kTiles)[warp] = out;
+            };
             const bool more = t + 1 < ntl;
             const double2 *np = tile_base(more ? t + 1 : t) + off;
 #pragma unroll
@@ -296,6 +308,7 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
                 };
                 wait_slot(q0);
                 if (failed) break;
+                if (s == 0) post();
                 unsigned char *sl = ring + (q0 % SLOTS) * kSlot + col;
                 unsigned re[2][kDigits], im[2][kDigits];
 #pragma unroll
@@ -376,8 +389,8 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
             }
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             double2 *base = tile_base(t);
-            const int ex = exps[(t & 3) * 128 + m] - 1022 + a.su - (68 - C::SH);
-            const bool plain = odd[t & 3] != 0;
+            const int ex = exps[(t % kTiles) * 128 + m] - 1022 + a.su - (68 - C::SH);
+            const bool plain = odd[t % kTiles] != 0;
             if (plain && h == 0) plain_tile<MODE>(a, base, ew * 32 + lane);
             const unsigned acc = tmem + (unsigned)(ab * 256) + ((unsigned)(32 * sub) << 16);
             if (!plain) {
@@ -418,11 +431,6 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
                 }
             }
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-            if (h == UNITS - 1) {
-                // every reading warp is past its look at the tile's flag before it is taken back
-                asm volatile("bar.sync 1, 256;\n" ::: "memory");
-                if (ew == 0 && lane == 0) odd[t & 3] = 0;
-            }
             __syncwarp();
             if (lane == 0) mbar_arrive(&accempty[ab]);
         }
