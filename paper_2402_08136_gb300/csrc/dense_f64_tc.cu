@@ -80,7 +80,7 @@ struct Cfg {
     static constexpr int SH = RED > 64 ? 13 : 12;
     static constexpr int BBYTES = UNITS * KS * kBlock;
     static constexpr int STAGE = kEpiWarps * 2048;
-    static constexpr int SMEM = BBYTES + SLOTS * kSlot + STAGE + kTiles * (128 * 4 + 8) + 8 * (2 * SLOTS + 5) + 16;
+    static constexpr int SMEM = BBYTES + SLOTS * kSlot + STAGE + kTiles * (128 * 4 + 8) + 8 * (2 * SLOTS + 6) + 16;
 };
 
 struct Args {
@@ -113,8 +113,9 @@ __device__ __forceinline__ void tmem_ld4(unsigned addr, float (&v)[4]) {
 }
 
 // A tile in FP64 by the 256 reading threads, U's columns in the plain kernels' order: all outputs before any store.
+// False, and nothing stored, when the wait for the other reading warps at `computed` ran out.
 template <int MODE>
-__device__ __noinline__ void plain_tile(const Args &a, double2 *base, int t) {
+__device__ __noinline__ bool plain_tile(const Args &a, double2 *base, int t, uint64_t *computed, unsigned parity) {
     using C = Cfg<MODE>;
     constexpr int D = C::D, TPG = 256 >> C::GB, OUT = D / TPG;  // threads per group, outputs per thread
     const int g = t & ((1 << C::GB) - 1), part = t >> C::GB;
@@ -135,9 +136,12 @@ __device__ __noinline__ void plain_tile(const Args &a, double2 *base, int t) {
         }
         y[o] = s;
     }
-    asm volatile("bar.sync 1, 256;\n" ::: "memory");
+    __syncwarp();
+    if ((t & 31) == 0) mbar_arrive(computed);
+    if (!__all_sync(~0u, mbar_wait(computed, parity))) return false;
 #pragma unroll 1
     for (int o = 0; o < OUT; o++) base[a.amp[part * OUT + o]] = y[o];
+    return true;
 }
 
 // z, or for a row that only scales its amplitude the value at p scaled.
@@ -194,8 +198,8 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
     int *exps = reinterpret_cast<int *>(stage + C::STAGE);  // [kTiles][128 rows]
     uint64_t *odd = reinterpret_cast<uint64_t *>(exps + kTiles * 128);  // [kTiles], a byte per loading warp: plain_tile if any is set
     uint64_t *full = odd + kTiles;
-    uint64_t *empty = full + SLOTS, *accfull = empty + SLOTS, *accempty = accfull + 2, *drain = accempty + 2;
-    unsigned *tslot = reinterpret_cast<unsigned *>(drain + 1);
+    uint64_t *empty = full + SLOTS, *accfull = empty + SLOTS, *accempty = accfull + 2, *drain = accempty + 2, *computed = drain + 1;
+    unsigned *tslot = reinterpret_cast<unsigned *>(computed + 1);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     for (int i = tid; i < C::BBYTES / 16; i += kThreads) reinterpret_cast<uint4 *>(sm)[i] = a.dig[i];
@@ -209,6 +213,7 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
             mbar_init(&accempty[i], kEpiWarps);
         }
         mbar_init(drain, 1);
+        mbar_init(computed, kEpiWarps);
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tslot)), "r"(512u)
@@ -378,6 +383,7 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
             if ((sr >> b) & 1) off += a.grp[b];
         off += (sub & 1) ? a.grp[PARTS ? 4 : 5] : 0;
         off += (sub & 2) ? a.grp[PARTS ? 5 : 6] : 0;
+        unsigned plains = 0;  // tiles so far that took plain_tile: the parity of `computed`
         for (long long u = 0; u < ntl * UNITS && !failed; u++) {
             const long long t = u / UNITS;
             const int h = (int)(u % UNITS), ab = (int)(u & 1);
@@ -391,7 +397,10 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
             double2 *base = tile_base(t);
             const int ex = exps[(t % kTiles) * 128 + m] - 1022 + a.su - (68 - C::SH);
             const bool plain = odd[t % kTiles] != 0;
-            if (plain && h == 0) plain_tile<MODE>(a, base, ew * 32 + lane);
+            if (plain && h == 0 && !plain_tile<MODE>(a, base, ew * 32 + lane, computed, plains++ & 1)) {
+                failed = true;
+                break;
+            }
             const unsigned acc = tmem + (unsigned)(ab * 256) + ((unsigned)(32 * sub) << 16);
             if (!plain) {
 #pragma unroll 1
