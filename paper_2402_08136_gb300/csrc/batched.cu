@@ -237,7 +237,7 @@ __device__ bool fourier_fx(double2 *x, unsigned N, int f0, int K, const int4 *W,
         const int E = (int)(m >> 20);
         if (m) {
             bad |= E > kMaxExp;
-            atomicMax(&ex[column(i)], E);
+            atomicMax(&ex[column(i)], max(E, 1));  // subnormals have exponent 0, which stands for a column of zeros
         } else {
             bad |= (__double2loint(z.x) | __double2loint(z.y)) != 0;
         }
