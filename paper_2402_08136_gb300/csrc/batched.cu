@@ -206,10 +206,16 @@ __device__ __forceinline__ V cmulb(V a, V b) {
     return r;
 }
 
-// A twiddle table's entry: complex128 tables hold the integers of the fixed-point passes
-// (dft_fx.cuh), 2^60 (c + i s) in halves.
-__device__ __forceinline__ float2 unit_root(const float2 *t, unsigned i) { return t[i]; }
-__device__ __forceinline__ double2 unit_root(const double2 *t, unsigned i) {
+// complex128 passes that run in fixed point have their tables as integers (dft_fx.cuh): 2^60 (c + i s) in halves.
+// Narrower fields and twiddles on the inputs stay in FP64, with FP64 tables.
+constexpr int kFxMinK = 5;
+__host__ __device__ __forceinline__ bool fixed_tables(int K, int twmode) { return K >= kFxMinK && twmode != 1; }
+
+// A twiddle table's entry.  An FP64 stage reads integers only where a column of a fixed-point pass is out of its
+// range (below 2^-60 off, under the 2^-53 that the stage rounds to).
+__device__ __forceinline__ float2 unit_root(const float2 *t, unsigned i, bool) { return t[i]; }
+__device__ __forceinline__ double2 unit_root(const double2 *t, unsigned i, bool fixed) {
+    if (!fixed) return t[i];
     const int4 e = reinterpret_cast<const int4 *>(t)[i];
     const long long c = ((long long)e.x << 32) + e.y, s = ((long long)e.z << 32) + e.w;
     return make_double2(dftk::fx::to_double(c, -60), dftk::fx::to_double(s, -60));
@@ -221,7 +227,7 @@ __device__ __forceinline__ double2 unit_root(const double2 *t, unsigned i) {
 // column (the other qubits fixed) gets its own exponent ex[]: 57 bits before the first five stages, and, for
 // wider fields, again before the rest (gr[]: the growth in between).  On return x holds integers, column c in
 // units of 2^(ex[c] - 1079).  False, x as it was, when a column is outside the fixed-point range.
-constexpr int kFxMinK = 5, kFxMaxCols = 256;
+constexpr int kFxMaxCols = 256;
 template <int NT>
 __device__ bool fourier_fx(double2 *x, unsigned N, int f0, int K, const int4 *W, bool walsh, int *ex, int tid) {
     using namespace dftk::fx;
@@ -316,15 +322,16 @@ __device__ void op_fourier(V *psi, int n, const BOp &op, const V *data, unsigned
     const unsigned N = 1u << n, fmask = ((1u << K) - 1u) << f0;
     const V *W = data + op.data;
     const int twmode = walsh ? 0 : op.t[1];
+    const bool fixed = fixed_tables(K, twmode);
     const int ns = op.nreg, s0 = op.t[0], hT = op.t[3];
     const V *Tlo = data + op.data2, *Thi = Tlo + (1u << hT);
     const unsigned smask = (1u << ns) - 1u, tmask = (1u << hT) - 1u;
     auto tw = [&](unsigned i, unsigned y) -> V {  // exp(s 2 pi i w y / 2^(K+ns))
         const unsigned q = ((i >> s0) & smask) * y;
-        return cmulb(unit_root(Tlo, q & tmask), unit_root(Thi, q >> hT));
+        return cmulb(unit_root(Tlo, q & tmask, fixed), unit_root(Thi, q >> hT, fixed));
     };
     if constexpr (sizeof(V) == 16 && CS == 1) {
-        if (shared && K >= kFxMinK && (N >> K) <= kFxMaxCols && twmode != 1) {
+        if (shared && fixed && (N >> K) <= kFxMaxCols) {
             const int4 *W4 = reinterpret_cast<const int4 *>(W), *lo4 = reinterpret_cast<const int4 *>(Tlo),
                        *hi4 = reinterpret_cast<const int4 *>(Thi);
             if (fourier_fx<NT>(psi, N, f0, K, W4, walsh, ex, (int)vt)) {
@@ -375,7 +382,7 @@ __device__ void op_fourier(V *psi, int n, const BOp &op, const V *data, unsigned
                 psi[i0[e]] = V{a[e].x + b[e].x, a[e].y + b[e].y};
                 if (!walsh) {
                     const unsigned r = (i0[e] >> f0) & rmask;
-                    if (r) d = cmulb(d, unit_root(W, r << (K - 1 - j)));
+                    if (r) d = cmulb(d, unit_root(W, r << (K - 1 - j), fixed));
                 }
                 psi[i0[e] | bit] = d;
             }
@@ -417,12 +424,13 @@ __device__ void op_fourier_tiled(V *g, int n, const BOp &op, const V *data, int 
     const unsigned ntile = 1u << (n - K - L);
     const V *W = data + op.data;
     const int twmode = walsh ? 0 : op.t[1];
+    const bool fixed = fixed_tables(K, twmode);
     const int ns = op.nreg, s0 = op.t[0], hT = op.t[3];
     const V *Tlo = data + op.data2, *Thi = Tlo + (1u << hT);
     const unsigned smask = (1u << ns) - 1u, tmask = (1u << hT) - 1u;
     auto tw = [&](unsigned i, unsigned y) -> V {
         const unsigned q = ((i >> s0) & smask) * y;
-        return cmulb(unit_root(Tlo, q & tmask), unit_root(Thi, q >> hT));
+        return cmulb(unit_root(Tlo, q & tmask, fixed), unit_root(Thi, q >> hT, fixed));
     };
     auto gidx = [&](unsigned o, unsigned j) -> unsigned {  // tile o, local index j = lane + (y << L)
         const unsigned olo = o & ((1u << mid) - 1u), ohi = o >> mid;
@@ -438,7 +446,7 @@ __device__ void op_fourier_tiled(V *g, int n, const BOp &op, const V *data, int 
         }
         __syncthreads();
         if constexpr (sizeof(V) == 16) {
-            if (K >= kFxMinK && (1u << L) <= kFxMaxCols && twmode != 1 &&
+            if (fixed && (1u << L) <= kFxMaxCols &&
                 fourier_fx<NT>(sm, TN, L, K, reinterpret_cast<const int4 *>(W), walsh, ex, tid)) {
                 const longlong2 *v = reinterpret_cast<const longlong2 *>(sm);
                 for (unsigned j = tid; j < TN; j += NT) {
@@ -463,7 +471,7 @@ __device__ void op_fourier_tiled(V *g, int n, const BOp &op, const V *data, int 
                 sm[i0] = V{a.x + b.x, a.y + b.y};
                 if (!walsh) {
                     const unsigned r = (i0 >> L) & rmask;
-                    if (r) d = cmulb(d, unit_root(W, r << (K - 1 - jj)));
+                    if (r) d = cmulb(d, unit_root(W, r << (K - 1 - jj), fixed));
                 }
                 sm[i0 | bit] = d;
             }
@@ -998,7 +1006,7 @@ bool encode(const Op &op, int dtype, std::vector<unsigned char> &data, BOp &b) {
             b.t[2] = (signed char)op.sign;
             b.t[3] = (signed char)((K + ns) / 2);  // the split dft_tables uses
             b.data2 = (unsigned)(el + W.size());
-            if (dtype == QSIM_C128) {  // the same tables as integers (dft_fx.cuh), 16 bytes an entry too
+            if (dtype == QSIM_C128 && batch::fixed_tables(K, b.t[1])) {  // as integers, 16 bytes an entry too
                 std::vector<int> fixed;
                 dft_fixed_tables(op, fixed);
                 const unsigned char *p = reinterpret_cast<const unsigned char *>(fixed.data());
