@@ -576,8 +576,10 @@ __device__ void run_op(typename C2<R>::T *psi, int n, const BOp &op, const typen
             const Rr Cs = d[0].x;
             // complex128, clock register right below the top qubit: the 2^c0 pairs of a clock value share its
             // rotation, so each lane of a warp computes that of one of 32 clock values (a division and a square
-            // root in FP64 for every pair took as long as three passes); with a pair per thread or less, each its own
-            if (sizeof(V) == 16 && cnt > (unsigned)kThreads && tq == n - 1 && op.c0 + op.nreg == n - 1) {
+            // root in FP64 for every pair took as long as three passes); with a pair per thread or less, or so few clock
+            // values that one warp would hold them all, each its own (96 circuits of 10 qubits, 16 values: 95.8 us a run
+            // on one warp, 88.0 with a rotation per pair; 64 values: 255 us per pair, 250 on two warps)
+            if (sizeof(V) == 16 && cnt > (unsigned)kThreads && (cnt >> op.c0) >= 64u && tq == n - 1 && op.c0 + op.nreg == n - 1) {
                 const unsigned rows = cnt >> op.c0, lane = vt & 31u;
                 for (unsigned b0 = (vt >> 5) * 32u; b0 < rows; b0 += kThreads) {
                     const unsigned raw = b0 + lane;
