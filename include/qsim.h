@@ -401,8 +401,9 @@ int hhl_readout(const void *state, int dtype, const hhl_circuit *h, void *stream
  * ends the structured HHL circuit), else by a reduction pass after it.  Device-only, so it can be captured into a CUDA graph.  hhl_readout_sums is
  * hhl_readout taking those partials instead of reducing the state again; the state must not
  * have changed since the hhl_run_sums that wrote sums_device.  Its device scratch comes from a
- * memory pool of the library's own (up to 64 MiB kept per device until the process ends); on a
- * stream of its own it also waits for work already enqueued on the default stream.
+ * memory pool of the library's own (up to 64 MiB kept per device until the process ends).
+ * It follows earlier work on its own stream; when hhl_run_sums of the same h has been captured,
+ * also the latest replay of that graph, on whichever stream.
  * Errors: EINVAL, ENOMEM, ECUDA. */
 #define QSIM_READOUT_SUMS_DOUBLES 4096
 int hhl_run_sums(void *state, int dtype, const hhl_circuit *h, const qsim_circuit *c, void *stream,

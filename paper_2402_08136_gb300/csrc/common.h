@@ -3,6 +3,7 @@
 
 #include <complex>
 #include <cstdint>
+#include <memory>
 #include <mutex>
 #include <stdexcept>
 #include <string>
@@ -15,6 +16,7 @@
 namespace qsim {
 
 using cd = std::complex<double>;
+struct ReplayMark;  // kernels.cu
 
 // Error carrying a status code; converted to a return value at the C boundary.
 struct Error : std::runtime_error {
@@ -131,7 +133,9 @@ struct qsim_circuit {
     std::vector<qsim::Op> ops;      // executable list (built lazily for unfused circuits)
     bool ops_ready = false;
     qsim::DeviceBlob blob[2];       // [0] complex64 matrices, [1] complex128 matrices
-    std::mutex mu;                  // guards ops/blob lazy construction
+    std::mutex mu;                  // guards ops/blob lazy construction, marks
+    // events inside captured runs of this circuit: kept as long as the tables that such a graph reads
+    std::vector<std::shared_ptr<qsim::ReplayMark>> marks;
     ~qsim_circuit();                // releases the device copies (kernels.cu)
 };
 
@@ -142,6 +146,8 @@ struct hhl_circuit {
     int n_total_formula = 0;
     std::vector<qsim::cd> b_pad;  // normalized, padded to 2^nb
     qsim_circuit circ;
+    mutable std::mutex mark_mu;  // guards mark
+    mutable std::shared_ptr<qsim::ReplayMark> mark;  // set once a run with readout sums has been captured
 };
 
 namespace qsim {
@@ -157,6 +163,10 @@ void circuit_info(const qsim_circuit *c, qsim_circuit_info *out);
 // of the final state (buf[0] = P, then P partials, the first half over the lower half of the
 // state): written by the last operation's kernel when it can, else by a reduction after it
 void apply_ops(void *state, int n, int dtype, qsim_circuit *c, void *stream, int live = -1, double *sums = nullptr);
+// after a run with sums on a stream under capture: an event into the graph, recorded by every replay
+void mark_replays(const hhl_circuit *h, qsim_circuit *c, void *stream);
+// the stream waits for the latest replay of h's marked runs on this device, if there are any
+void after_replays(const hhl_circuit *h, void *stream);
 // final readout from such a buffer: sums[3] and the (ancilla = 1, clock = 0) slice on the host
 void readout_device_sums(const void *state, int dtype, int n, int nb, void *stream, const double *buf,
                          double sums[3], cd *slice);

@@ -528,6 +528,7 @@ int hhl_run_sums(void *state, int dtype, const hhl_circuit *h, const qsim_circui
         QSIM_REQUIRE(g->n == h->n, "circuit and HHL problem disagree on the qubit count");
         launch_prepare_state(state, h->n, dtype, h->b_pad.data(), h->nb, stream, h->nb);
         apply_ops(state, h->n, dtype, const_cast<qsim_circuit *>(g), stream, h->nb, sums_device);
+        mark_replays(h, const_cast<qsim_circuit *>(g), stream);
     });
 }
 
@@ -538,6 +539,7 @@ int hhl_readout_sums(const void *state, int dtype, const hhl_circuit *h, const d
         QSIM_REQUIRE(dtype == QSIM_C64 || dtype == QSIM_C128, "dtype must be QSIM_C64 or QSIM_C128");
         double sums[3];
         std::vector<cd> slice((size_t)1 << h->nb);
+        after_replays(h, stream);
         readout_device_sums(state, dtype, h->n, h->nb, stream, sums_device, sums, slice.data());
         readout_finish(h, sums, slice, x_out, x_state_out, stats);
     });

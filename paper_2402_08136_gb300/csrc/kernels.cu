@@ -1613,28 +1613,60 @@ void readout_device(const void *state, int dtype, int n, int nb, int m, void *st
     fetch_readout(out, dtype, slice_len, st, sums, slice);
 }
 
-// A readout on a stream of its own comes after what is already enqueued on the device's default stream, where the
-// run it reads may have been replayed (allocating from the default pool used to take long enough for that).
-static void after_default_stream(cudaStream_t st) {
+// A captured run with readout sums may be replayed on another stream than its readout is called on, and the library
+// does not see the replay.  An event inside the graph, recorded by each replay, lets the readout wait for the run it
+// reads and for nothing else.  The event lives as long as the problem or a circuit whose graph holds it.
+struct ReplayMark {
+    std::mutex mu;
+    std::map<int, cudaEvent_t> event;  // by device
+    ~ReplayMark() {
+        for (auto &e : event) cudaEventDestroy(e.second);
+    }
+};
+
+void mark_replays(const hhl_circuit *h, qsim_circuit *c, void *stream) {
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (st == nullptr || st == cudaStreamLegacy) return;
-    // a blocking stream under capture forbids touching the default stream (the query does not disturb it)
-    if (cudaStreamIsCapturing(cudaStreamLegacy, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {  // the default stream while another one is under capture
         cudaGetLastError();
         return;
     }
-    cudaEvent_t ev = nullptr;
-    CUDA_OK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
-    cudaError_t e = cudaEventRecord(ev, cudaStreamLegacy);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ev, 0);
-    cudaEventDestroy(ev);
-    CUDA_OK(e);
+    if (cap != cudaStreamCaptureStatusActive) return;
+    std::shared_ptr<ReplayMark> mark;
+    {
+        std::lock_guard<std::mutex> lk(h->mark_mu);
+        if (!h->mark) h->mark = std::make_shared<ReplayMark>();
+        mark = h->mark;
+    }
+    {
+        std::lock_guard<std::mutex> lk(c->mu);
+        if (std::find(c->marks.begin(), c->marks.end(), mark) == c->marks.end()) c->marks.push_back(mark);
+    }
+    int dev = 0;
+    CUDA_OK(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lk(mark->mu);
+    cudaEvent_t &ev = mark->event[dev];
+    if (ev == nullptr) CUDA_OK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+    CUDA_OK(cudaEventRecordWithFlags(ev, st, cudaEventRecordExternal));
+}
+
+void after_replays(const hhl_circuit *h, void *stream) {
+    std::shared_ptr<ReplayMark> mark;
+    {
+        std::lock_guard<std::mutex> lk(h->mark_mu);
+        mark = h->mark;
+    }
+    if (!mark) return;
+    int dev = 0;
+    CUDA_OK(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lk(mark->mu);
+    const auto it = mark->event.find(dev);
+    if (it != mark->event.end() && it->second) CUDA_OK(cudaStreamWaitEvent(static_cast<cudaStream_t>(stream), it->second, 0));
 }
 
 void readout_device_sums(const void *state, int dtype, int n, int nb, void *stream, const double *buf,
                          double sums[3], cd *slice) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    after_default_stream(st);
     const size_t slice_len = (size_t)1 << nb;
     const long long off = 1ll << (n - 1);  // ancilla = 1 (the top qubit), clock = 0
     const ReadoutScratch scratch(4 * 8 + slice_len * 2 * real_size(dtype), true, st);
