@@ -107,8 +107,8 @@ struct Op {
     std::vector<int> tc_pads;
     size_t dev_off_tcw = 0;
     // complex128 dense op that runs as exact digit products on the tensor cores (dense_f64.cu; its
-    // digits at dev_off_tc[1]): entries of U are below 2^f64_su, bit r of f64_diag: row and column r
-    // are zero off the diagonal
+    // digits at dev_off_tc[1]): bit r of f64_diag: row and column r
+    // are zero off the diagonal; entries of the other rows are below 2^f64_su
     bool has_f64 = false;
     bool f64_tc = false;  // ... with the digits laid out for tcgen05 (dense_f64_tc.cu)
     int f64_su = 0;

@@ -27,7 +27,8 @@
 //
 // Not all gates take this form (dense_f64_applies): those with mostly zero rows keep the FP64
 // kernels, which are exact on permutations; rows that only scale their own amplitude (the padding of
-// an eigenvector matrix, a controlled gate written as a dense one) are computed in FP64 on the way out.
+// an eigenvector matrix, a controlled gate written as a dense one) are computed in FP64 on the way out, and
+// neither those amplitudes nor their entries count in the scales of the others.
 // A tile with a group that is not finite, or whose largest exponent is far from 1, is computed in
 // the plain FP64 form by the same warp (plain_tile).
 //
@@ -204,6 +205,16 @@ __global__ void __launch_bounds__(Cfg<K, REALU>::THREADS, 1) dense_f64_kernel(co
 #pragma unroll
         for (int i = 0; i < NT; i++) {
             char *tb = base + a.tile[i], *ob = tb + out_lane;
+            bool finite = true;
+            if (a.diag) {  // amplitudes that are only scaled take no part in the products or in their scale
+                const unsigned long long mine = a.diag >> q;
+#pragma unroll
+                for (int e = 0; e < EPL; e++)
+                    if ((mine >> (4 * (REALU ? e : e / 2))) & 1ull) {
+                        finite = finite && mag_bits(x[i][e]) < 0x7ff00000u;
+                        x[i][e] = 0.0;
+                    }
+            }
             // exponent of each column's largest value: over the quad, or for narrow gates (RF, k < 3)
             // over the amplitudes that share the bits from k on
             unsigned m0 = 0, m1 = 0;
@@ -225,7 +236,7 @@ __global__ void __launch_bounds__(Cfg<K, REALU>::THREADS, 1) dense_f64_kernel(co
                 m1 = m0;
             }
             const int E0 = m0 ? (int)(m0 >> 20) : 1023, E1 = m1 ? (int)(m1 >> 20) : 1023;
-            bool fits = E0 >= kMinExp && E0 <= kMaxExp && E1 >= kMinExp && E1 <= kMaxExp;
+            bool fits = finite && E0 >= kMinExp && E0 <= kMaxExp && E1 >= kMinExp && E1 <= kMaxExp;
             if (m0 == 0 || m1 == 0) {  // all zero, or denormals whose high words are 0
                 unsigned low = 0;
 #pragma unroll
@@ -348,7 +359,7 @@ static void pack_digits(const Op &op, int su, unsigned char *out) {
     const int k = (int)op.targets.size(), D0 = 1 << k;
     unsigned short *o = reinterpret_cast<unsigned short *>(out);
     auto entry = [&](int r, int c) -> cd {  // group bits from k on: identity
-        if ((r >> k) != (c >> k)) return cd(0.0, 0.0);
+        if ((r >> k) != (c >> k) || ((op.f64_diag >> (r & (D0 - 1))) & 1ull)) return cd(0.0, 0.0);
         return op.U[(size_t)(r & (D0 - 1)) * D0 + (c & (D0 - 1))];
     };
     const int tabs = C::TABS == 3 ? 2 : 1;
@@ -468,18 +479,17 @@ size_t dense_f64_blob_bytes(const Op &op) {
     return n;
 }
 
-// exponent of U's scale: every entry is below 2^su in magnitude
-static int scale_of(const Op &op) {
-    double top = 0.0;
-    for (const cd &u : op.U) top = std::max(top, std::max(std::fabs(u.real()), std::fabs(u.imag())));
-    int e = 0;
-    std::frexp(top, &e);  // top = f 2^e, f in [1/2, 1)
-    return e;
-}
-
+// f64_su: exponent of U's scale, every entry of a row that is not only scaled is below 2^su in magnitude
 void dense_f64_scale(Op &op) {
-    op.f64_su = scale_of(op);
+    const int D = 1 << (int)op.targets.size();
     op.f64_diag = diagonal_rows(op);
+    double top = 0.0;
+    for (int r = 0; r < D; r++)
+        for (int c = 0; c < D && !((op.f64_diag >> r) & 1ull); c++) {
+            const cd &u = op.U[(size_t)r * D + c];
+            top = std::max(top, std::max(std::fabs(u.real()), std::fabs(u.imag())));
+        }
+    std::frexp(top, &op.f64_su);  // top = f 2^su, f in [1/2, 1)
 }
 
 void dense_f64_pack(const Op &op, unsigned char *out) {

@@ -258,6 +258,17 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
         for (long long t = 0; t < ntl && !failed; t++) {
             int Er[ITEMS], Ei[ITEMS];
             bool out = false;  // a group is outside the fixed-point range
+            if (a.diag) {      // amplitudes that are only scaled take no part in the products or in their scale
+                const unsigned long long mine = a.diag >> kc;
+#pragma unroll
+                for (int it = 0; it < ITEMS; it++)
+#pragma unroll
+                    for (int e = 0; e < EPT; e++)
+                        if ((mine >> (4 * e)) & 1ull) {
+                            out |= max(mag_bits(x[it][e].x), mag_bits(x[it][e].y)) >= 0x7ff00000u;
+                            x[it][e] = make_double2(0.0, 0.0);
+                        }
+            }
 #pragma unroll
             for (int it = 0; it < ITEMS; it++) {
                 unsigned mr = 0, mi = 0, low = 0;
@@ -522,6 +533,7 @@ template <int MODE>
 static void pack(const Op &op, unsigned char *out) {
     using C = Cfg<MODE>;
     const double scale = std::ldexp(1.0, 62 - op.f64_su);
+    auto entry = [&](int r, int c) { return (op.f64_diag >> r) & 1ull ? cd(0.0, 0.0) : op.U[(size_t)r * C::D + c]; };
     for (int h = 0; h < C::UNITS; h++)
         for (int ks = 0; ks < C::KS; ks++) {
             unsigned short *blk = reinterpret_cast<unsigned short *>(out + (size_t)(h * C::KS + ks) * kBlock);
@@ -531,10 +543,10 @@ static void pack(const Op &op, unsigned char *out) {
                     double u;
                     if (C::PARTS) {
                         const int step = MODE == C6 ? ks >> 1 : ks;
-                        const cd z = op.U[(size_t)(32 * h + n) * C::D + kc + 4 * (4 * step + r)];
+                        const cd z = entry(32 * h + n, kc + 4 * (4 * step + r));
                         u = MODE == C6 && (ks & 1) ? z.imag() : z.real();
                     } else {
-                        const cd z = op.U[(size_t)(16 * h + (n >> 1)) * C::D + kc + 4 * (2 * ks + (r >> 1))];
+                        const cd z = entry(16 * h + (n >> 1), kc + 4 * (2 * ks + (r >> 1)));
                         if (n & 1) u = (r & 1) ? z.real() : z.imag();
                         else u = (r & 1) ? -z.imag() : z.real();
                     }
