@@ -7,6 +7,7 @@
 #include <mutex>
 #include <stdexcept>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -106,13 +107,22 @@ struct Op {
     // dev_off_tcw: the widened form's blob (complex64 device data)
     std::vector<int> tc_pads;
     size_t dev_off_tcw = 0;
-    // complex128 dense op that runs as exact digit products on the tensor cores (dense_f64.cu; its
-    // digits at dev_off_tc[1]): bit r of f64_diag: row and column r
-    // are zero off the diagonal; entries of the other rows are below 2^f64_su
+    // complex128 dense op that runs as exact digit products on the tensor cores (dense_f64_plan; its digits at
+    // dev_off_tc[1]).  f64_U: the matrix applied when that is not U (empty: U), in FP64 and transposed at f64_ut_off;
+    // output r is then its row s for the pairs (r, s) of f64_moves, row r for the others.  Bit r of f64_diag: entry (r, r)
+    // is multiplied in FP64.  What is left has its rows and columns scaled by 2^-f64_row[r] 2^-f64_col[c] and is then
+    // below 2^f64_su; f64_sh: bits dropped from a sum; f64_rows: bytes and thresholds of the rows, f64_check: groups are
+    // tested with them
     bool has_f64 = false;
     bool f64_tc = false;  // ... with the digits laid out for tcgen05 (dense_f64_tc.cu)
-    int f64_su = 0;
+    bool f64_check = false;
+    int f64_su = 0, f64_sh = 0, f64_reach = 0;
     unsigned long long f64_diag = 0;
+    std::vector<cd> f64_U;
+    std::vector<std::pair<int, int>> f64_moves;
+    std::vector<int> f64_row, f64_col;  // kNoEntries: nothing left in it
+    std::vector<unsigned char> f64_rows;
+    size_t f64_ut_off = 0;
     int sparse_w = 0;  // complex128 dense op of at most this many nonzeros a row (dense_sparse.cu; entries at dev_off_tc[1])
     bool real_u = false;        // OP_DENSE: every entry of U is real (SIMT kernels use 2 FMAs per entry)
 };
@@ -211,10 +221,13 @@ bool launch_dense_tc_real7(void *state, int n, const std::vector<int> &targets, 
                            const void *Bdev, int sms, cudaStream_t st, double *sums = nullptr, int hi_bit = 0,
                            bool *sums_written = nullptr);
 // dense_f64.cu: complex128 dense gates as exact digit products on the tensor cores
-bool dense_f64_applies(const Op &op);
+bool dense_f64_plan(Op &op);  // sets op.f64_*; false: the gate is not one of them
 size_t dense_f64_blob_bytes(const Op &op);
-void dense_f64_scale(Op &op);  // sets op.f64_su, op.f64_diag
 void dense_f64_pack(const Op &op, unsigned char *out);
+cd dense_f64_entry(const Op &op, int r, int c);
+void dense_f64_pack_scales(const Op &op, unsigned char *out);  // two doubles a row
+unsigned long long dense_f64_beside(const Op &op);
+void launch_dense_f64_moves(void *state, int n, const Op &op, int sms, cudaStream_t st);
 // Ut: U in FP64, transposed; false (nothing launched) when the state has too few groups
 bool launch_dense_f64(void *state, int n, const Op &op, const void *dig, const void *Ut, int sms, cudaStream_t st);
 // dense_f64_tc.cu: the same products with tcgen05 for wide gates (4 and 5 targets complex, 6 targets real or

@@ -22,14 +22,16 @@
 // units, put the sums together, and pass the amplitudes through shared memory so that a warp's store covers
 // 4 amplitudes of 8 groups (the lowest targets and free qubits: whole lines).  Roles meet at mbarriers only,
 // every wait is bounded, tensor memory is freed after the last MMA has completed (as in dense_tc.cu).
-// A tile with a group outside the fixed-point range is computed in FP64 by the reading warps (plain_tile).
+// Groups outside the fixed-point range, or whose sums would lose more than an FP64 sum (dense_f64_plan), are marked and
+// computed in FP64 by the reading warps (plain_groups).
 //
 // 26 qubits, dense_f64.cu's form -> this one, TB/s: 4 targets 2.42 -> 3.54, 5 1.40 -> 2.9, 6 0.77 -> 1.63, 6 with a real U
 // 1.57 -> 2.8.  What bounds it: issue slots for splitting and joining the digits (0.59 instructions a clock and
 // scheduler at 4 targets, 0.50 at 5; the tensor pipe at 21 to 39 %); at 6 complex targets the MMAs and the joining take turns, as tensor
 // memory holds one tile's two units and no more.  The FP64 pipe is at 17 to 37 %: its last
-// conversion only, scaled rows apart, whose products sit behind a branch of their own (as predicated instructions
-// they passed the pipe for every row: 69 % of it).
+// conversion only, apart from rows with an entry left to FP64, which have a function of their own (with them in the
+// main path the pipe was 69 % busy).  Testing the groups of an eigenvector matrix with many small entries, and marking
+// them one by one, costs a 27-qubit solve 13.27 -> 13.67 ms (with tiles marked as a whole some systems took 17 ms and more).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -56,7 +58,7 @@ constexpr int kThreads = (kMmaWarp + 4) * 32;  // the issuing warp's group of fo
 constexpr int kProdRegs = 128, kEpiRegs = 80, kMmaRegs = 56;
 constexpr int kSlot = kDigits * 4096;  // one K-step of a tile: 8 digits x 128 rows x 16 FP16
 constexpr int kBlock = 8192;           // U's digits of one unit and K-step: 256 rows x 16 FP16
-// Slots of what the loading warps tell the reading ones about a tile (exponents, odd marks).  Tile t is written once
+// Slots of what the loading warps tell the reading ones about a tile (exponents, marked groups).  Tile t is written once
 // its first K-step has a ring slot, so the MMAs of the K-step SLOTS before it are complete, and they had waited for
 // the unit two before theirs to be read: tile t - 4 with 4 targets (2 tiles in the ring, 2 in tensor memory), tile
 // t - 2 in the other modes.  Every earlier tile has been read when slot t mod 4 is written.
@@ -76,20 +78,21 @@ struct Cfg {
     static constexpr int EPT = MODE == C4 ? 4 : MODE == C5 ? 8 : 16;  // amplitudes per item: every fourth
     static constexpr int STEP = PARTS ? 4 : 2;            // amplitudes per item and K-step
     static constexpr int RED = MODE == C4 ? 32 : MODE == C6 ? 128 : 64;
-    static constexpr bool BIAS = RED <= 32;
-    static constexpr int SH = RED > 64 ? 13 : 12;
+    static constexpr int BIAS = RED <= 32 ? kept_shift(RED) : 0;
     static constexpr int BBYTES = UNITS * KS * kBlock;
     static constexpr int STAGE = kEpiWarps * 2048;
-    static constexpr int SMEM = BBYTES + SLOTS * kSlot + STAGE + kTiles * (128 * 4 + 8) + 8 * (2 * SLOTS + 6) + 16;
+    static constexpr int ROWS = rows_bytes(D);
+    static constexpr int SMEM = BBYTES + SLOTS * kSlot + STAGE + ROWS + kTiles * (128 * 4 + 8 * ITEMS) + 8 * (2 * SLOTS + 5) + 16;
 };
 
 struct Args {
     double2 *psi;
     const uint4 *dig;
     const double2 *Ut;
+    const double2 *vw;  // as in dense_f64.cu
     long long ntiles;
-    unsigned long long cmask, diag;
-    int su, nfix;
+    unsigned long long cmask, diag, beside;
+    int su, sh, check, reach, nfix;  // as in dense_f64.cu
     int fix[kMaxFix];   // ascending: targets, controls, group bits inside a tile
     long long amp[64];  // offset (in amplitudes) of amplitude a of a group
     long long grp[7];   // ... of group bit b of a tile
@@ -112,61 +115,73 @@ __device__ __forceinline__ void tmem_ld4(unsigned addr, float (&v)[4]) {
     for (int i = 0; i < 4; i++) v[i] = __uint_as_float(r[i]);
 }
 
-// A tile in FP64 by the 256 reading threads, U's columns in the plain kernels' order: all outputs before any store.
-// False, and nothing stored, when the wait for the other reading warps at `computed` ran out.
+// The marked groups of a tile, in FP64: a warp takes every eighth (with 4 targets every eighth pair) and stores a group
+// when all of its outputs are computed.  A lane has rows lane and lane + 32, U's columns in the plain kernels' order.
 template <int MODE>
-__device__ __noinline__ bool plain_tile(const Args &a, double2 *base, int t, uint64_t *computed, unsigned parity) {
+__device__ __noinline__ void plain_groups(const Args &a, double2 *base, const uint64_t *marks, int ew, int lane) {
     using C = Cfg<MODE>;
-    constexpr int D = C::D, TPG = 256 >> C::GB, OUT = D / TPG;  // threads per group, outputs per thread
-    const int g = t & ((1 << C::GB) - 1), part = t >> C::GB;
-    for (int b = 0; b < C::GB; b++)
-        if ((g >> b) & 1) base += a.grp[b];
-    double2 y[OUT];
-#pragma unroll 1
-    for (int o = 0; o < OUT; o++) {
-        const int r = part * OUT + o;
-        double2 s = make_double2(0.0, 0.0);
-#pragma unroll 1
-        for (int c = 0; c < D; c++) {
-            const double2 x = base[a.amp[c]], u = a.Ut[c * D + r];
-            s.x = fma(u.x, x.x, s.x);
-            if (MODE != R6) s.x = fma(-u.y, x.y, s.x);
-            s.y = fma(u.x, x.y, s.y);
-            if (MODE != R6) s.y = fma(u.y, x.x, s.y);
+    constexpr int D = C::D, L = D < 32 ? D : 32, ROWS = D / L;  // lanes per group, rows per lane
+    int n = (32 / L) * ew + lane / L, r = lane % L;  // the warp's next mark, counted over the tile
+    for (int w = 0; w < C::ITEMS; w++) {
+        uint64_t m = marks[w];
+        int left = __popcll(m);
+        while (__any_sync(~0u, n < left)) {
+            const bool mine = n < left;
+            uint64_t k = m;
+            for (int i = 0; i < n && mine; i++) k &= k - 1;  // the n-th set bit
+            const int g = 64 * w + (mine ? __ffsll((long long)k) - 1 : 0);
+            double2 *p = base, y[ROWS];
+            for (int b = 0; b < C::GB; b++)
+                if ((g >> b) & 1) p += a.grp[b];
+#pragma unroll
+            for (int o = 0; o < ROWS; o++) y[o] = make_double2(0.0, 0.0);
+            if (mine)
+#pragma unroll 2
+                for (int c = 0; c < D; c++) {
+                    const double2 x = p[a.amp[c]];
+#pragma unroll
+                    for (int o = 0; o < ROWS; o++) {
+                        const double2 u = __ldg(a.Ut + c * D + r + 32 * o);
+                        y[o].x = fma(u.x, x.x, y[o].x);
+                        if (MODE != R6) y[o].x = fma(-u.y, x.y, y[o].x);
+                        y[o].y = fma(u.x, x.y, y[o].y);
+                        if (MODE != R6) y[o].y = fma(u.y, x.x, y[o].y);
+                    }
+                }
+            __syncwarp();
+            if (mine)
+#pragma unroll
+                for (int o = 0; o < ROWS; o++) p[a.amp[r + 32 * o]] = y[o];
+            if (mine) n += kEpiWarps * (32 / L);
         }
-        y[o] = s;
+        n -= left;
     }
-    __syncwarp();
-    if ((t & 31) == 0) mbar_arrive(computed);
-    if (!__all_sync(~0u, mbar_wait(computed, parity))) return false;
-#pragma unroll 1
-    for (int o = 0; o < OUT; o++) base[a.amp[part * OUT + o]] = y[o];
-    return true;
 }
 
-// z, or for a row that only scales its amplitude the value at p scaled.
+// Where a diagonal entry is left to FP64: the sum z of the rest plus its product with the value at p.
 template <int MODE>
 __device__ __noinline__ double2 scaled_row(const Args &a, int row, const double2 *p, double2 z) {
-    if ((a.diag >> row) & 1ull) {
-        const double2 w = __ldg(a.Ut + row * Cfg<MODE>::D + row), o = *p;
-        z.x = w.x * o.x;
-        z.y = w.x * o.y;
-        if (MODE != R6) {
-            z.x = fma(-w.y, o.y, z.x);
-            z.y = fma(w.y, o.x, z.y);
-        }
+    const double2 w = __ldg(a.Ut + row * Cfg<MODE>::D + row), o = *p;
+    const double rest = (a.beside >> row) & 1ull ? __ldg(a.vw + row).y : 0.0;
+    z.x = fma(w.x, o.x, rest * z.x);
+    z.y = fma(w.x, o.y, rest * z.y);
+    if (MODE != R6) {
+        z.x = fma(-w.y, o.y, z.x);
+        z.y = fma(w.y, o.x, z.y);
     }
     return z;
 }
-// The amplitudes of 8 columns from the warp's stage to their places: lane (4 lowest amplitudes, 8 groups).
-template <int MODE, bool DIAG>
-__device__ __forceinline__ void store_body(const Args &a, const unsigned char *st, double2 *at, int h, int s, int lane) {
+// The amplitudes of 8 columns from the warp's stage to their places: lane (4 lowest amplitudes, 8 groups).  SPEC: some
+// rows have a diagonal entry left to FP64, or some of the warp's groups (bits of skip) are not stored here.
+template <int MODE, bool SPEC>
+__device__ __forceinline__ void store_body(const Args &a, const unsigned char *st, double2 *at, int h, int s, int lane, unsigned skip) {
     using C = Cfg<MODE>;
     const int sa = lane & 3, sr = lane >> 2;
 #pragma unroll
     for (int i = 0; i < 4; i++) {
         double2 z, *p = at;
         int row;
+        if (SPEC && ((skip >> (8 * (C::PARTS ? i & 1 : i) + sr)) & 1u)) continue;
         if (C::PARTS) {
             const int g = 8 * (i & 1) + sr, c = sa + 4 * (i >> 1);
             z = *reinterpret_cast<const double2 *>(st + g * 128 + ((c ^ (g & 7)) * 16));
@@ -178,13 +193,13 @@ __device__ __forceinline__ void store_body(const Args &a, const unsigned char *s
             row = 16 * h + 4 * s + sa;
             p += ((i & 1) ? a.grp[3] : 0) + ((i & 2) ? a.grp[4] : 0) + a.amp[16 * h + 4 * s];
         }
-        if (DIAG) z = scaled_row<MODE>(a, row, p, z);
+        if (SPEC && ((a.diag >> row) & 1ull)) z = scaled_row<MODE>(a, row, p, z);
         __stcs(p, z);
     }
 }
 template <int MODE>
-__device__ __noinline__ void store_diag(const Args &a, const unsigned char *st, double2 *at, int h, int s, int lane) {
-    store_body<MODE, true>(a, st, at, h, s, lane);
+__device__ __noinline__ void store_spec(const Args &a, const unsigned char *st, double2 *at, int h, int s, int lane, unsigned skip) {
+    store_body<MODE, true>(a, st, at, h, s, lane, skip);
 }
 
 template <int MODE>
@@ -195,14 +210,17 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
     extern __shared__ __align__(1024) unsigned char sm[];
     unsigned char *ring = sm + C::BBYTES;
     unsigned char *stage = ring + SLOTS * kSlot;
-    int *exps = reinterpret_cast<int *>(stage + C::STAGE);  // [kTiles][128 rows]
-    uint64_t *odd = reinterpret_cast<uint64_t *>(exps + kTiles * 128);  // [kTiles], a byte per loading warp: plain_tile if any is set
-    uint64_t *full = odd + kTiles;
-    uint64_t *empty = full + SLOTS, *accfull = empty + SLOTS, *accempty = accfull + 2, *drain = accempty + 2, *computed = drain + 1;
-    unsigned *tslot = reinterpret_cast<unsigned *>(computed + 1);
+    unsigned char *rows = stage + C::STAGE;                        // bytes and thresholds of U's rows
+    int *exps = reinterpret_cast<int *>(rows + C::ROWS);           // [kTiles][128 rows]
+    uint64_t *marks = reinterpret_cast<uint64_t *>(exps + kTiles * 128);  // [kTiles][ITEMS], a bit per group: in FP64
+    uint64_t *full = marks + kTiles * ITEMS;
+    uint64_t *empty = full + SLOTS, *accfull = empty + SLOTS, *accempty = accfull + 2, *drain = accempty + 2;
+    unsigned *tslot = reinterpret_cast<unsigned *>(drain + 1);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     for (int i = tid; i < C::BBYTES / 16; i += kThreads) reinterpret_cast<uint4 *>(sm)[i] = a.dig[i];
+    if (a.check)
+        for (int i = tid; i < C::ROWS / 16; i += kThreads) reinterpret_cast<uint4 *>(rows)[i] = a.dig[C::BBYTES / 16 + i];
     if (tid == 0) {
         for (int i = 0; i < SLOTS; i++) {
             mbar_init(&full[i], kProdWarps);
@@ -213,7 +231,6 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
             mbar_init(&accempty[i], kEpiWarps);
         }
         mbar_init(drain, 1);
-        mbar_init(computed, kEpiWarps);
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tslot)), "r"(512u)
@@ -257,16 +274,17 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
         const unsigned col = (unsigned)((kc >> 1) * 128 + (kc & 1) * 8);
         for (long long t = 0; t < ntl && !failed; t++) {
             int Er[ITEMS], Ei[ITEMS];
-            bool out = false;  // a group is outside the fixed-point range
-            if (a.diag) {      // amplitudes that are only scaled take no part in the products or in their scale
+            bool out[ITEMS] = {};  // the group is outside the fixed-point range, or its sums would lose too much
+            if (a.diag) {      // amplitudes with a diagonal entry of their own: scaled to what else is in their column, or 0
                 const unsigned long long mine = a.diag >> kc;
 #pragma unroll
                 for (int it = 0; it < ITEMS; it++)
 #pragma unroll
                     for (int e = 0; e < EPT; e++)
                         if ((mine >> (4 * e)) & 1ull) {
-                            out |= max(mag_bits(x[it][e].x), mag_bits(x[it][e].y)) >= 0x7ff00000u;
-                            x[it][e] = make_double2(0.0, 0.0);
+                            out[it] |= max(mag_bits(x[it][e].x), mag_bits(x[it][e].y)) >= 0x7ff00000u;
+                            const double v = (a.beside >> (kc + 4 * e)) & 1ull ? __ldg(a.vw + kc + 4 * e).x : 0.0;
+                            x[it][e] = make_double2(x[it][e].x * v, x[it][e].y * v);
                         }
             }
 #pragma unroll
@@ -277,7 +295,8 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
                     mr = max(mr, mag_bits(x[it][e].x));
                     mi = max(mi, mag_bits(x[it][e].y));
                 }
-                if (MODE != R6) mr = mi = max(mr, mi);  // one exponent for both parts where they mix
+                const unsigned ml = max(mr, mi);
+                if (MODE != R6) mr = mi = ml;  // one exponent for both parts where they mix
                 mr = max(mr, __shfl_xor_sync(~0u, mr, 8));
                 mr = max(mr, __shfl_xor_sync(~0u, mr, 16));
                 if (MODE == R6) {
@@ -294,9 +313,25 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
                         if (!mag_bits(x[it][e].x)) low |= (unsigned)__double2loint(x[it][e].x);
                         if (!mag_bits(x[it][e].y)) low |= (unsigned)__double2loint(x[it][e].y);
                     }
-                out |= Er[it] < kMinExp || Er[it] > kMaxExp || Ei[it] < kMinExp || Ei[it] > kMaxExp || low;
+                out[it] |= Er[it] < kMinExp || Er[it] > kMaxExp || Ei[it] < kMinExp || Ei[it] > kMaxExp || low;
+                if (a.check) {  // by the larger part of an amplitude
+                    const int E = PARTS ? max(mr ? Er[it] : 0, mi ? Ei[it] : 0) : Er[it];
+                    const bool zero = mr == 0 && mi == 0;
+                    if (!__all_sync(~0u, (int)(ml >> 20) >= E - a.reach || zero)) {
+                        unsigned m[EPT];
+#pragma unroll
+                        for (int e = 0; e < EPT; e++) m[e] = max(mag_bits(x[it][e].x), mag_bits(x[it][e].y));
+                        out[it] |= !rows_fit_of<C::D, 8, 16>(m, E, zero, kc, a.diag, rows);
+                    }
+                }
             }
-            out = __any_sync(~0u, out);
+            unsigned char mark[ITEMS];  // of the warp's 8 groups
+#pragma unroll
+            for (int it = 0; it < ITEMS; it++) {
+                unsigned m = __ballot_sync(~0u, out[it]);
+                m |= m >> 16;
+                mark[it] = (unsigned char)(m | m >> 8);
+            }
             auto post = [&] {  // after the wait for the tile's first ring slot (see kTiles)
                 int *ex = exps + (t % kTiles) * 128;
                 if (kc == 0) {
@@ -310,7 +345,10 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
                         }
                     }
                 }
-                if (lane == 0) reinterpret_cast<unsigned char *>(odd + t % kTiles)[warp] = out;
+                if (lane == 0)
+#pragma unroll
+                    for (int it = 0; it < ITEMS; it++)
+                        reinterpret_cast<unsigned char *>(marks + (t % kTiles) * ITEMS + it)[warp] = mark[it];
             };
             const bool more = t + 1 < ntl;
             const double2 *np = tile_base(more ? t + 1 : t) + off;
@@ -394,7 +432,6 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
             if ((sr >> b) & 1) off += a.grp[b];
         off += (sub & 1) ? a.grp[PARTS ? 4 : 5] : 0;
         off += (sub & 2) ? a.grp[PARTS ? 5 : 6] : 0;
-        unsigned plains = 0;  // tiles so far that took plain_tile: the parity of `computed`
         for (long long u = 0; u < ntl * UNITS && !failed; u++) {
             const long long t = u / UNITS;
             const int h = (int)(u % UNITS), ab = (int)(u & 1);
@@ -406,14 +443,12 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
             }
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             double2 *base = tile_base(t);
-            const int ex = exps[(t % kTiles) * 128 + m] - 1022 + a.su - (68 - C::SH);
-            const bool plain = odd[t % kTiles] != 0;
-            if (plain && h == 0 && !plain_tile<MODE>(a, base, ew * 32 + lane, computed, plains++ & 1)) {
-                failed = true;
-                break;
-            }
+            const int ex = exps[(t % kTiles) * 128 + m] - 1022 + a.su - 68 + a.sh;
+            const uint64_t *mt = marks + (t % kTiles) * ITEMS;
+            const unsigned skip = PARTS ? (unsigned)(mt[0] >> (16 * sub)) & 0xffffu : (unsigned)(mt[ITEMS > 1 ? sub >> 1 : 0] >> (32 * (sub & 1)));
+            if (h == 0 && (mt[0] | mt[ITEMS - 1]) != 0) plain_groups<MODE>(a, base, mt, ew, lane);
             const unsigned acc = tmem + (unsigned)(ab * 256) + ((unsigned)(32 * sub) << 16);
-            if (!plain) {
+            if (skip != (PARTS ? 0xffffu : ~0u)) {
 #pragma unroll 1
                 for (int s = 2 * (ew >> 2); s < 2 * (ew >> 2) + 2; s++) {  // columns 8 s .. 8 s + 7 of the unit
                     __syncwarp();  // the previous step's amplitudes have been read
@@ -428,8 +463,8 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
                         for (int c = 0; c < 4; c++) {
                             float w[kDigits];
 #pragma unroll
-                            for (int d = 0; d < kDigits; d++) w[d] = C::BIAS ? v[d][c] + kBiasF : v[d][c];
-                            y[c] = join<C::BIAS, C::SH>(w, ex);
+                            for (int d = 0; d < kDigits; d++) w[d] = C::BIAS > 0 ? v[d][c] + kBiasF : v[d][c];
+                            y[c] = join<C::BIAS>(w, a.sh, ex);
                         }
                         if (PARTS) {  // row (group, part): parts of 8 amplitudes
                             const int g = lane >> 1;
@@ -444,10 +479,9 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
                         }
                     }
                     __syncwarp();
-                    // gates with rows that only scale their amplitude take a function of their own: as a condition
-                    // here its FP64 operations are predicated and pass through the FP64 pipe for every amplitude
-                    if (a.diag) store_diag<MODE>(a, st, base + off, h, s, lane);
-                    else store_body<MODE, false>(a, st, base + off, h, s, lane);
+                    // a function of its own: with the FP64 products as a condition here the FP64 pipe was 69 % busy
+                    if (a.diag || skip) store_spec<MODE>(a, st, base + off, h, s, lane, skip);
+                    else store_body<MODE, false>(a, st, base + off, h, s, lane, 0u);
                 }
             }
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
@@ -533,7 +567,7 @@ template <int MODE>
 static void pack(const Op &op, unsigned char *out) {
     using C = Cfg<MODE>;
     const double scale = std::ldexp(1.0, 62 - op.f64_su);
-    auto entry = [&](int r, int c) { return (op.f64_diag >> r) & 1ull ? cd(0.0, 0.0) : op.U[(size_t)r * C::D + c]; };
+    auto entry = [&](int r, int c) { return dense_f64_entry(op, r, c); };
     for (int h = 0; h < C::UNITS; h++)
         for (int ks = 0; ks < C::KS; ks++) {
             unsigned short *blk = reinterpret_cast<unsigned short *>(out + (size_t)(h * C::KS + ks) * kBlock);
@@ -557,6 +591,8 @@ static void pack(const Op &op, unsigned char *out) {
                     }
                 }
         }
+    std::memcpy(out + C::BBYTES, op.f64_rows.data(), C::ROWS);
+    dense_f64_pack_scales(op, out + C::BBYTES + C::ROWS);
 }
 
 static int mode_of(const Op &op) {
@@ -600,7 +636,7 @@ size_t dense_f64_tc_blob_bytes(const Op &op, int n) {
     using namespace f64tc;
     size_t bytes = 0;
     int gb = 0;
-#define QSIM_BYTES(M) bytes = Cfg<M>::BBYTES, gb = Cfg<M>::GB
+#define QSIM_BYTES(M) bytes = Cfg<M>::BBYTES + Cfg<M>::ROWS + 16 * Cfg<M>::D, gb = Cfg<M>::GB
     QSIM_F64TC_SWITCH(mode_of(op), QSIM_BYTES)
 #undef QSIM_BYTES
     return n - (int)(op.targets.size() + op.controls.size()) >= gb + 7 ? bytes : 0;
@@ -617,8 +653,8 @@ bool launch_dense_f64_tc(void *state, int n, const Op &op, const void *dig, cons
     using namespace f64tc;
     const int mode = mode_of(op);
     if (mode < 0) return false;
-    int gb = 0;
-#define QSIM_GB(M) gb = Cfg<M>::GB
+    int gb = 0, vw = 0;
+#define QSIM_GB(M) gb = Cfg<M>::GB, vw = Cfg<M>::BBYTES + Cfg<M>::ROWS
     QSIM_F64TC_SWITCH(mode, QSIM_GB)
 #undef QSIM_GB
     Args a;
@@ -634,9 +670,14 @@ bool launch_dense_f64_tc(void *state, int n, const Op &op, const void *dig, cons
     a.psi = static_cast<double2 *>(state);
     a.dig = static_cast<const uint4 *>(dig);
     a.Ut = static_cast<const double2 *>(Ut);
+    a.vw = reinterpret_cast<const double2 *>(static_cast<const unsigned char *>(dig) + vw);
     a.ntiles = 1ll << ((int)fr.size() - gb);
     a.diag = op.f64_diag;
+    a.beside = dense_f64_beside(op);
     a.su = op.f64_su;
+    a.sh = op.f64_sh;
+    a.check = op.f64_check ? 1 : 0;
+    a.reach = op.f64_reach;
     const int k = (int)op.targets.size();
     for (int v = 0; v < (1 << k); v++)
         for (int b = 0; b < k; b++)

@@ -1150,9 +1150,8 @@ std::vector<unsigned char> pack_device_blob(qsim_circuit *c, int dtype) {
                 dense_tc_pack(6, UW, blob.data() + op.dev_off_tcw);
             }
             if (dtype == QSIM_C128) {
-                op.has_f64 = dense_f64_applies(op);
+                op.has_f64 = dense_f64_plan(op);
                 if (op.has_f64) {
-                    dense_f64_scale(op);
                     const size_t tcb = dense_f64_tc_blob_bytes(op, c->n);
                     op.f64_tc = tcb > 0;
                     align_blob(blob);
@@ -1160,6 +1159,13 @@ std::vector<unsigned char> pack_device_blob(qsim_circuit *c, int dtype) {
                     blob.resize(blob.size() + (tcb ? tcb : dense_f64_blob_bytes(op)));
                     if (tcb) dense_f64_tc_pack(op, blob.data() + op.dev_off_tc[slot]);
                     else dense_f64_pack(op, blob.data() + op.dev_off_tc[slot]);
+                    op.f64_ut_off = op.dev_off[slot];
+                    if (!op.f64_U.empty()) {
+                        align_blob(blob);
+                        op.f64_ut_off = blob.size();
+                        for (int cc = 0; cc < D; cc++)
+                            for (int r = 0; r < D; r++) put_complex(blob, dtype, op.f64_U[(size_t)r * D + cc]);
+                    }
                 } else if ((op.sparse_w = sparse_width(op)) > 0) {
                     align_blob(blob);
                     op.dev_off_tc[slot] = blob.size();
@@ -1422,9 +1428,11 @@ void apply_ops(void *state, int n, int dtype, qsim_circuit *c, void *stream, int
                         break;
                 }
                 if (dtype == QSIM_C128 && op.has_f64 &&
-                    (op.f64_tc ? launch_dense_f64_tc : launch_dense_f64)(state, w, op, base + op.dev_off_tc[slot], dptr,
-                                                                         num_sms(), st))
+                    (op.f64_tc ? launch_dense_f64_tc : launch_dense_f64)(state, w, op, base + op.dev_off_tc[slot],
+                                                                         base + op.f64_ut_off, num_sms(), st)) {
+                    if (!op.f64_moves.empty()) launch_dense_f64_moves(state, w, op, num_sms(), st);
                     break;
+                }
                 if (dtype == QSIM_C128 && op.sparse_w > 0) {
                     launch_sparse(state, w, op, base + op.dev_off_tc[slot], dptr, num_sms(), st);
                     break;
