@@ -242,7 +242,7 @@ void dense_f64_clear_error();
 // not sparse); any gate of 3..7 targets on a state of at most 8 groups (false: more groups)
 int sparse_width(const Op &op);
 void sparse_pack(const Op &op, std::vector<unsigned char> &blob);
-void launch_sparse(void *state, int n, const Op &op, const void *ell, const void *Ut, int sms, cudaStream_t st);
+bool launch_sparse(void *state, int n, const Op &op, const void *ell, const void *Ut, int sms, cudaStream_t st);
 bool launch_group(void *state, int n, int dtype, const Op &op, const void *Ut, cudaStream_t st);
 // batched.cu: plan (host image) / instantiate (device tables) / launch / results, for the pool
 struct BatchImage;

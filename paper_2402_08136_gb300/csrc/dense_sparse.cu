@@ -194,10 +194,16 @@ void sparse_pack(const Op &op, std::vector<unsigned char> &blob) {
     blob.insert(blob.end(), p, p + col.size() * sizeof(int));
 }
 
-void launch_sparse(void *state, int n, const Op &op, const void *ell, const void *Ut, int sms, cudaStream_t st) {
+// False (nothing launched): a real U with half of a row nonzero on 2^20 amplitudes or more.  The row form is bound by the
+// reads of its entries there, as long for a real U as for a complex one, and the tiled kernels' real form is ahead: 25
+// qubits, 1..5 targets 428, 650, 1081, 1945, 3715 us here and 270, 517, 1027, 1785, 3520 there (20 qubits: 29.5, 38.5, 54, 87,
+// 151 and 27, 36, 54, 84, 148; 18 qubits: 19, 22, 26, 34, 51 and 20, 22, 27, 36, 54).  With fewer entries, or a complex U, the
+// row form is never behind.
+bool launch_sparse(void *state, int n, const Op &op, const void *ell, const void *Ut, int sms, cudaStream_t st) {
     sparse::Args a;
     std::memset(&a, 0, sizeof(a));
     const int K = (int)op.targets.size(), D = 1 << K, avail = n - (int)op.controls.size();
+    if (op.real_u && 2 * op.sparse_w == D && avail >= 20) return false;
     a.psi = static_cast<double2 *>(state);
     a.W = op.sparse_w;
     a.K = K;
@@ -239,6 +245,7 @@ void launch_sparse(void *state, int n, const Op &op, const void *ell, const void
     sparse::sparse_kernel<<<(int)grid, sparse::kThreads, smem, st>>>(a);
     cuda_check("sparse_kernel");
     note_launches(1, QSIM_KERNEL_DENSE_SIMT);
+    return true;
 }
 
 // At most 8 groups (a CTA each): larger states fill the tiled kernels' warps.

@@ -1433,10 +1433,9 @@ void apply_ops(void *state, int n, int dtype, qsim_circuit *c, void *stream, int
                     if (!op.f64_moves.empty()) launch_dense_f64_moves(state, w, op, num_sms(), st);
                     break;
                 }
-                if (dtype == QSIM_C128 && op.sparse_w > 0) {
-                    launch_sparse(state, w, op, base + op.dev_off_tc[slot], dptr, num_sms(), st);
+                if (dtype == QSIM_C128 && op.sparse_w > 0 &&
+                    launch_sparse(state, w, op, base + op.dev_off_tc[slot], dptr, num_sms(), st))
                     break;
-                }
                 if (dtype == QSIM_C128 && launch_group(state, w, dtype, op, dptr, st)) break;
                 run_dense(state, w, dtype, op, dptr, st);
                 break;
