@@ -773,9 +773,12 @@ void launch_dense_f64_moves(void *state, int n, const Op &op, int sms, cudaStrea
     note_launches(1, QSIM_KERNEL_DENSE_SIMT);
 }
 
-// Returns false when the state is too small for the kernel's tiles (the plain kernels take it).
+// Returns false when the state is too small for the kernel's tiles, or for a real 1-target gate (Hadamard, RY) on 2^18
+// amplitudes or more: its 2 multiply-adds a real cost FP64 less than splitting and joining cost here (25 qubits 260 us
+// there, 288 here; 27 qubits 1000, 1115; 18 qubits 9.8, 11.4; below, 16 qubits, 9.9, 8.8).  The plain kernels take both.
 bool launch_dense_f64(void *state, int n, const Op &op, const void *dig, const void *Ut, int sms, cudaStream_t st) {
     const int k = (int)op.targets.size(), K = f64::width_of(op);
+    if (k == 1 && op.real_u && n - (int)op.controls.size() >= 18) return false;
     int tb = 0, gb = 0, warps = 0;  // warps: of a full chip
 #define QSIM_F64_BITS(KK, R) tb = f64::Cfg<KK, R>::TB, gb = f64::Cfg<KK, R>::GB, warps = sms * f64::Cfg<KK, R>::THREADS / 32
     QSIM_F64_SWITCH(op, QSIM_F64_BITS)

@@ -195,3 +195,14 @@ def test_rows_that_hardly_mix(qs, k, n, real):
                 elif what == "one":
                     psi[rows(n, t) != col[0]] = 0
                 check(qs, psi, n, t, U)
+
+
+@pytest.mark.parametrize("n,ctl,digits", [(17, 0, True), (18, 0, False), (18, 1, True), (19, 1, False)])
+def test_real_single_targets(qs, n, ctl, digits):
+    """Both sides of the rule that leaves real 1-target gates to FP64 (2^18 amplitudes, controls apart)."""
+    rng = np.random.default_rng(n + ctl)
+    for U in (np.array([[1, 1], [1, -1]]) / 2 ** 0.5, haar(rng, 2, True)):
+        q = [int(v) for v in rng.permutation(n)]
+        before = qs.qsim_launch_counts()["dense_tc"]
+        check(qs, synth.gaussian_state_np(n, n), n, q[:1], U.astype(np.complex128), q[1:1 + ctl])
+        assert (qs.qsim_launch_counts()["dense_tc"] > before) == digits
