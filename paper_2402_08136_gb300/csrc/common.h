@@ -118,7 +118,7 @@ struct Op {
     bool f64_check = false;
     int f64_su = 0, f64_sh = 0, f64_reach = 0;
     unsigned long long f64_diag = 0;
-    std::vector<cd> f64_U;
+    std::vector<cd> f64_U, f64_left;  // (f64_left, f64_rows: until they are packed)
     std::vector<std::pair<int, int>> f64_moves;
     std::vector<int> f64_row, f64_col;  // kNoEntries: nothing left in it
     std::vector<unsigned char> f64_rows;
@@ -224,7 +224,6 @@ bool launch_dense_tc_real7(void *state, int n, const std::vector<int> &targets, 
 bool dense_f64_plan(Op &op);  // sets op.f64_*; false: the gate is not one of them
 size_t dense_f64_blob_bytes(const Op &op);
 void dense_f64_pack(const Op &op, unsigned char *out);
-cd dense_f64_entry(const Op &op, int r, int c);
 void dense_f64_pack_scales(const Op &op, unsigned char *out);  // two doubles a row
 unsigned long long dense_f64_beside(const Op &op);
 void launch_dense_f64_moves(void *state, int n, const Op &op, int sms, cudaStream_t st);

@@ -144,9 +144,13 @@ __device__ __forceinline__ void put(const Args &a, int row, char *at, double2 y)
     if (SPEC && ((a.diag >> row) & 1ull)) {
         const int r = row & ((1 << a.k) - 1);
         const double2 u = __ldg(a.Ut + (r << a.k) + r), x = *p;
-        const double w = (a.beside >> row) & 1ull ? __ldg(a.vw + r).y : 0.0;
-        y.x = fma(u.x, x.x, w * y.x);
-        y.y = fma(u.x, x.y, w * y.y);
+        if (K >= 4 && ((a.beside >> row) & 1ull)) {
+            const double w = __ldg(a.vw + r).y;
+            y.x *= w;
+            y.y *= w;
+        }
+        y.x = fma(u.x, x.x, y.x);  // without other entries in the row the sum is 0
+        y.y = fma(u.x, x.y, y.y);
         if (!a.real_u) {
             y.x = fma(-u.y, x.y, y.x);
             y.y = fma(u.y, x.x, y.y);
@@ -220,24 +224,27 @@ __global__ void __launch_bounds__(Cfg<K, REALU>::THREADS, 1) dense_f64_kernel(co
 #pragma unroll
         for (int i = 0; i < NT; i++) {
             char *tb = base + a.tile[i], *ob = tb + out_lane;
-            bool finite = true;
-            if (SPEC && a.diag) {  // amplitudes with a diagonal entry of their own: scaled to what else is in their column, or 0
-                const unsigned long long mine = a.diag >> q;
+            if (SPEC && K >= 4 && a.beside) {  // amplitudes with a diagonal entry of their own, scaled to the rest of their column
 #pragma unroll
                 for (int e = 0; e < EPL; e++) {
-                    const int c = 4 * (REALU ? e : e / 2);
-                    if ((mine >> c) & 1ull) {
-                        finite = finite && mag_bits(x[i][e]) < 0x7ff00000u;
-                        x[i][e] = (a.beside >> (q + c)) & 1ull ? x[i][e] * __ldg(a.vw + q + c).x : 0.0;
-                    }
+                    const int c = q + 4 * (REALU ? e : e / 2);
+                    if ((a.beside >> c) & 1ull) x[i][e] *= __ldg(a.vw + c).x;
                 }
             }
+            // amplitudes without such a rest do not count: U's digits are 0 in their columns, whatever theirs are
+            const unsigned long long alone = SPEC ? (a.diag & ~a.beside) >> q : 0ull;
+            unsigned all = 0;
+            auto mag = [&](int e) -> unsigned {
+                const unsigned m = mag_bits(x[i][e]);
+                all = max(all, m);
+                return SPEC && ((alone >> (4 * (REALU ? e : e / 2))) & 1ull) ? 0u : m;
+            };
             // exponent of each column's largest value: over the quad, or for narrow gates (RF, k < 3)
             // over the amplitudes that share the bits from k on
-            unsigned m0 = 0, m1 = 0, ml = 0;  // ml: of this lane
+            unsigned m0 = 0, m1 = 0, l0 = 0, l1 = 0;  // l0, l1: of this lane
             if constexpr (C::RF) {
-                m0 = max(mag_bits(x[i][0]), mag_bits(x[i][1]));
-                m1 = max(mag_bits(x[i][2]), mag_bits(x[i][3]));
+                m0 = l0 = max(mag(0), mag(1));
+                m1 = l1 = max(mag(2), mag(3));
                 m0 = max(m0, __shfl_xor_sync(~0u, m0, 1));
                 m1 = max(m1, __shfl_xor_sync(~0u, m1, 1));
                 if (a.k >= 2) {
@@ -247,14 +254,14 @@ __global__ void __launch_bounds__(Cfg<K, REALU>::THREADS, 1) dense_f64_kernel(co
                 if (a.k >= 3) m0 = m1 = max(m0, m1);
             } else {
 #pragma unroll
-                for (int e = 0; e < EPL; e++) m0 = max(m0, mag_bits(x[i][e]));
-                ml = m0;
+                for (int e = 0; e < EPL; e++) m0 = max(m0, mag(e));
+                l0 = m0;
                 m0 = max(m0, __shfl_xor_sync(~0u, m0, 1));
                 m0 = max(m0, __shfl_xor_sync(~0u, m0, 2));
                 m1 = m0;
             }
             const int E0 = m0 ? (int)(m0 >> 20) : 1023, E1 = m1 ? (int)(m1 >> 20) : 1023;
-            bool fits = finite && E0 >= kMinExp && E0 <= kMaxExp && E1 >= kMinExp && E1 <= kMaxExp;
+            bool fits = (!SPEC || all < 0x7ff00000u) && E0 >= kMinExp && E0 <= kMaxExp && E1 >= kMinExp && E1 <= kMaxExp;
             if (m0 == 0 || m1 == 0) {  // all zero, or denormals whose high words are 0
                 unsigned low = 0;
 #pragma unroll
@@ -263,8 +270,7 @@ __global__ void __launch_bounds__(Cfg<K, REALU>::THREADS, 1) dense_f64_kernel(co
             }
             if (SPEC && a.check) {
                 if constexpr (C::RF) {  // rows q and q + 4; the quad's amplitudes as bytes of two words
-                    unsigned w[2] = {mag_byte(max(mag_bits(x[i][0]), mag_bits(x[i][1])), E0) << (8 * q),
-                                     mag_byte(max(mag_bits(x[i][2]), mag_bits(x[i][3])), E1) << (8 * q)};
+                    unsigned w[2] = {mag_byte(l0, E0) << (8 * q), mag_byte(l1, E1) << (8 * q)};
 #pragma unroll
                     for (int h = 0; h < 2; h++) {
                         w[h] |= __shfl_xor_sync(~0u, w[h], 1);
@@ -274,11 +280,11 @@ __global__ void __launch_bounds__(Cfg<K, REALU>::THREADS, 1) dense_f64_kernel(co
                     fits = fits && (m0 == 0 || dot_bytes<2>(u + 2 * q, w, 0u) >= thr[q]) &&
                            (m1 == 0 || dot_bytes<2>(u + 2 * q + 8, w, 0u) >= thr[q + 4]);
                 } else {
-                    if (!__all_sync(~0u, (int)(ml >> 20) >= E0 - a.reach || m0 == 0)) {
+                    if (!__all_sync(~0u, (int)(l0 >> 20) >= E0 - a.reach || m0 == 0)) {
                         unsigned m[C::D / 4];
 #pragma unroll
                         for (int e = 0; e < C::D / 4; e++)
-                            m[e] = REALU ? mag_bits(x[i][e]) : max(mag_bits(x[i][2 * e]), mag_bits(x[i][2 * e + 1]));
+                            m[e] = REALU ? mag(e) : max(mag(2 * e), mag(2 * e + 1));
                         fits = rows_fit_of<C::D, 1, 2>(m, E0, m0 == 0, q, a.diag, rows) && fits;
                     }
                 }
@@ -429,7 +435,7 @@ static void pack_digits(const Op &op, int su, unsigned char *out) {
     const int k = (int)op.targets.size(), D0 = 1 << k;
     unsigned short *o = reinterpret_cast<unsigned short *>(out);
     auto entry = [&](int r, int c) -> cd {  // group bits from k on: identity
-        return (r >> k) == (c >> k) ? dense_f64_entry(op, r & (D0 - 1), c & (D0 - 1)) : cd(0.0, 0.0);
+        return (r >> k) == (c >> k) ? op.f64_left[(size_t)(r & (D0 - 1)) * D0 + (c & (D0 - 1))] : cd(0.0, 0.0);
     };
     const int tabs = C::TABS == 3 ? 2 : 1;
     const double scale = std::ldexp(1.0, 62 - su);
@@ -636,15 +642,6 @@ static bool scale(Op &op) {
     return true;
 }
 
-// Entry (r, c) as it is split into digits.
-cd dense_f64_entry(const Op &op, int r, int c) {
-    if (r == c && ((op.f64_diag >> r) & 1ull)) return cd(0.0, 0.0);
-    const cd u = f64::matrix(op)[((size_t)r << op.targets.size()) + c];
-    if (op.f64_diag == 0 || u == cd(0.0, 0.0)) return u;
-    const int e = -op.f64_row[r] - op.f64_col[c];
-    return cd(std::ldexp(u.real(), e), std::ldexp(u.imag(), e));
-}
-
 unsigned long long dense_f64_beside(const Op &op) {
     unsigned long long m = 0;
     for (size_t i = 0; i < op.f64_row.size(); i++)
@@ -679,11 +676,15 @@ bool dense_f64_plan(Op &op) {
     const int k = (int)op.targets.size(), D = 1 << k;
     separate(op);
     if (op.f64_moves.size() > f64::kMaxMoves || !scale(op)) return false;
+    op.f64_left = f64::matrix(op);  // as it is split into digits
     double sum = 0.0;
     for (int r = 0; r < D; r++) {
         double s = 0.0;
         for (int c = 0; c < D; c++) {
-            const cd u = dense_f64_entry(op, r, c);
+            cd &u = op.f64_left[(size_t)r * D + c];
+            if (r == c && ((op.f64_diag >> r) & 1ull)) u = 0.0;
+            const int er = op.f64_row[r], ec = op.f64_col[c];
+            if ((er != 0 || ec != 0) && u != cd(0.0, 0.0)) u = cd(std::ldexp(u.real(), -er - ec), std::ldexp(u.imag(), -er - ec));
             s += std::fabs(u.real()) + std::fabs(u.imag());
         }
         sum = std::max(sum, s);
@@ -697,6 +698,7 @@ bool dense_f64_plan(Op &op) {
     op.f64_rows.assign(f64::rows_bytes(DK), 0);
     unsigned *at = reinterpret_cast<unsigned *>(op.f64_rows.data() + DK * DK);
     int *from = reinterpret_cast<int *>(at + DK);
+    const double units = std::ldexp(1.0, 8 - op.f64_su);
     for (int r = 0; r < D; r++) {
         if (op.f64_row[r] == kNoEntries) continue;
         int nz = 0;
@@ -704,8 +706,8 @@ bool dense_f64_plan(Op &op) {
         unsigned lane[4] = {255, 255, 255, 255};
         for (int c = 0; c < D; c++) {
             if (op.f64_col[c] == kNoEntries) continue;
-            const cd u = dense_f64_entry(op, r, c);
-            const unsigned b = (unsigned)std::ldexp(size_of(u), 8 - op.f64_su);
+            const cd u = op.f64_left[(size_t)r * D + c];
+            const unsigned b = (unsigned)(size_of(u) * units);
             if (k >= 4) op.f64_rows[(size_t)r * D + (c & 3) * (D / 4) + (c >> 2)] = (unsigned char)b;
             for (int g = 0; k <= 3 && g < 8; g += D) op.f64_rows[(size_t)(g + r) * 8 + g + c] = (unsigned char)b;
             nz += u != cd(0.0, 0.0);

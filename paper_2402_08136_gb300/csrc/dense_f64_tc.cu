@@ -283,8 +283,12 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
                     for (int e = 0; e < EPT; e++)
                         if ((mine >> (4 * e)) & 1ull) {
                             out[it] |= max(mag_bits(x[it][e].x), mag_bits(x[it][e].y)) >= 0x7ff00000u;
-                            const double v = (a.beside >> (kc + 4 * e)) & 1ull ? __ldg(a.vw + kc + 4 * e).x : 0.0;
-                            x[it][e] = make_double2(x[it][e].x * v, x[it][e].y * v);
+                            if ((a.beside >> (kc + 4 * e)) & 1ull) {
+                                const double v = __ldg(a.vw + kc + 4 * e).x;
+                                x[it][e] = make_double2(x[it][e].x * v, x[it][e].y * v);
+                            } else {
+                                x[it][e] = make_double2(0.0, 0.0);
+                            }
                         }
             }
 #pragma unroll
@@ -567,7 +571,7 @@ template <int MODE>
 static void pack(const Op &op, unsigned char *out) {
     using C = Cfg<MODE>;
     const double scale = std::ldexp(1.0, 62 - op.f64_su);
-    auto entry = [&](int r, int c) { return dense_f64_entry(op, r, c); };
+    auto entry = [&](int r, int c) { return op.f64_left[(size_t)r * C::D + c]; };
     for (int h = 0; h < C::UNITS; h++)
         for (int ks = 0; ks < C::KS; ks++) {
             unsigned short *blk = reinterpret_cast<unsigned short *>(out + (size_t)(h * C::KS + ks) * kBlock);

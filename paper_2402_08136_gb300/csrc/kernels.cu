@@ -1166,6 +1166,8 @@ std::vector<unsigned char> pack_device_blob(qsim_circuit *c, int dtype) {
                         for (int cc = 0; cc < D; cc++)
                             for (int r = 0; r < D; r++) put_complex(blob, dtype, op.f64_U[(size_t)r * D + cc]);
                     }
+                    std::vector<cd>().swap(op.f64_left);
+                    std::vector<unsigned char>().swap(op.f64_rows);
                 } else if ((op.sparse_w = sparse_width(op)) > 0) {
                     align_blob(blob);
                     op.dev_off_tc[slot] = blob.size();
