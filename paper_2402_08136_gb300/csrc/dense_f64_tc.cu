@@ -116,36 +116,42 @@ __device__ __forceinline__ void tmem_ld4(unsigned addr, float (&v)[4]) {
 }
 
 // The marked groups of a tile, in FP64: a warp takes every eighth (with 4 targets every eighth pair) and stores a group
-// when all of its outputs are computed.  A lane has rows lane and lane + 32, U's columns in the plain kernels' order.
+// when all of its outputs are computed.  A lane has rows lane and lane + 32 and loads those amplitudes; U's columns come in
+// the plain kernels' order, the column's amplitude from its lane.
 template <int MODE>
-__device__ __noinline__ void plain_groups(const Args &a, double2 *base, const uint64_t *marks, int ew, int lane) {
+__device__ __noinline__ void plain_groups(const Args &a, double2 *base, uint64_t m0, uint64_t m1, int ew, int lane) {
     using C = Cfg<MODE>;
     constexpr int D = C::D, L = D < 32 ? D : 32, ROWS = D / L;  // lanes per group, rows per lane
     int n = (32 / L) * ew + lane / L, r = lane % L;  // the warp's next mark, counted over the tile
     for (int w = 0; w < C::ITEMS; w++) {
-        uint64_t m = marks[w];
-        int left = __popcll(m);
+        const uint64_t m = w ? m1 : m0;
+        const int left = __popcll(m);
         while (__any_sync(~0u, n < left)) {
             const bool mine = n < left;
             uint64_t k = m;
             for (int i = 0; i < n && mine; i++) k &= k - 1;  // the n-th set bit
             const int g = 64 * w + (mine ? __ffsll((long long)k) - 1 : 0);
-            double2 *p = base, y[ROWS];
+            double2 *p = base, x[ROWS], y[ROWS];
             for (int b = 0; b < C::GB; b++)
                 if ((g >> b) & 1) p += a.grp[b];
 #pragma unroll
-            for (int o = 0; o < ROWS; o++) y[o] = make_double2(0.0, 0.0);
-            if (mine)
-#pragma unroll 2
-                for (int c = 0; c < D; c++) {
-                    const double2 x = p[a.amp[c]];
+            for (int o = 0; o < ROWS; o++) {
+                x[o] = mine ? p[a.amp[r + 32 * o]] : make_double2(0.0, 0.0);
+                y[o] = make_double2(0.0, 0.0);
+            }
+#pragma unroll
+            for (int h = 0; h < ROWS; h++)
+#pragma unroll 4
+                for (int c = 0; c < L; c++) {  // amplitude c + 32 h, from its lane
+                    const double zx = __shfl_sync(~0u, x[h].x, c, L), zy = __shfl_sync(~0u, x[h].y, c, L);
 #pragma unroll
                     for (int o = 0; o < ROWS; o++) {
-                        const double2 u = __ldg(a.Ut + c * D + r + 32 * o);
-                        y[o].x = fma(u.x, x.x, y[o].x);
-                        if (MODE != R6) y[o].x = fma(-u.y, x.y, y[o].x);
-                        y[o].y = fma(u.x, x.y, y[o].y);
-                        if (MODE != R6) y[o].y = fma(u.y, x.x, y[o].y);
+                        const double2 *w = a.Ut + (c + 32 * h) * D + r + 32 * o;
+                        const double2 u = MODE == R6 ? make_double2(__ldg(&w->x), 0.0) : __ldg(w);
+                        y[o].x = fma(u.x, zx, y[o].x);
+                        if (MODE != R6) y[o].x = fma(-u.y, zy, y[o].x);
+                        y[o].y = fma(u.x, zy, y[o].y);
+                        if (MODE != R6) y[o].y = fma(u.y, zx, y[o].y);
                     }
                 }
             __syncwarp();
@@ -449,8 +455,8 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
             double2 *base = tile_base(t);
             const int ex = exps[(t % kTiles) * 128 + m] - 1022 + a.su - 68 + a.sh;
             const uint64_t *mt = marks + (t % kTiles) * ITEMS;
-            const unsigned skip = PARTS ? (unsigned)(mt[0] >> (16 * sub)) & 0xffffu : (unsigned)(mt[ITEMS > 1 ? sub >> 1 : 0] >> (32 * (sub & 1)));
-            if (h == 0 && (mt[0] | mt[ITEMS - 1]) != 0) plain_groups<MODE>(a, base, mt, ew, lane);
+            const uint64_t m0 = mt[0], m1 = ITEMS > 1 ? mt[ITEMS - 1] : 0;
+            const unsigned skip = PARTS ? (unsigned)(m0 >> (16 * sub)) & 0xffffu : (unsigned)((sub < 2 ? m0 : m1) >> (32 * (sub & 1)));
             const unsigned acc = tmem + (unsigned)(ab * 256) + ((unsigned)(32 * sub) << 16);
             if (skip != (PARTS ? 0xffffu : ~0u)) {
 #pragma unroll 1
@@ -491,6 +497,9 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(&accempty[ab]);
+            // behind the release, by another warp first for every tile: the FP64 pipe of one scheduler takes 9 us for a group
+            // of 6 targets with a real U, and the other warps and the MMAs go on meanwhile
+            if (h == UNITS - 1 && (m0 | m1) != 0) plain_groups<MODE>(a, base, m0, m1, (int)((ew - t) & (kEpiWarps - 1)), lane);
         }
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(kMmaRegs));
