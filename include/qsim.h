@@ -46,7 +46,12 @@ extern "C" {
 
 /* ---- state dtypes ---------------------------------------------------------------------- */
 #define QSIM_C64 1  /* complex64: FP32 state; gate arithmetic FP32 (dense k>=4 on tensor cores) */
-#define QSIM_C128 2 /* complex128: FP64 state; gate arithmetic exact to FP64 rounding or better   */
+#define QSIM_C128 2 /* complex128: FP64 state.  Dense gates: each output amplitude within the bound
+                     * of an FP64 sum of its own n products, n 2^-53 sum |u_rc| |x_c| (n = 2^k of k
+                     * targets, twice that for a complex matrix).  Fourier and Walsh-Hadamard passes:
+                     * each output within 8 (K + 2) 2^-53 2^(K/2) times the largest amplitude of
+                     * its column (the 2^K amplitudes that differ in the field), as an FP64 transform:
+                     * relative to that amplitude, not to the output.                           */
 
 typedef struct qsim_circuit qsim_circuit; /* gate list (unfused or fused)                       */
 typedef struct hhl_circuit hhl_circuit;   /* HHL problem + its unfused gate list                */

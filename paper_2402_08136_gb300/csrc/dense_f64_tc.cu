@@ -208,7 +208,9 @@ __device__ __noinline__ void store_spec(const Args &a, const unsigned char *st, 
     store_body<MODE, true>(a, st, at, h, s, lane, skip);
 }
 
-template <int MODE>
+// SPEC: gates with diagonal entries multiplied in FP64, or whose groups are tested (as instructions of the one kernel that
+// others pass by, 23 qubits: 4, 5, 6 real, 6 targets 87 106 111 185 us, without them 84 102 102 181).
+template <int MODE, bool SPEC>
 __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_constant__ Args a) {
     using C = Cfg<MODE>;
     constexpr int KS = C::KS, SLOTS = C::SLOTS, ITEMS = C::ITEMS, EPT = C::EPT, STEP = C::STEP, UNITS = C::UNITS;
@@ -225,7 +227,7 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     for (int i = tid; i < C::BBYTES / 16; i += kThreads) reinterpret_cast<uint4 *>(sm)[i] = a.dig[i];
-    if (a.check)
+    if (SPEC && a.check)
         for (int i = tid; i < C::ROWS / 16; i += kThreads) reinterpret_cast<uint4 *>(rows)[i] = a.dig[C::BBYTES / 16 + i];
     if (tid == 0) {
         for (int i = 0; i < SLOTS; i++) {
@@ -281,7 +283,7 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
         for (long long t = 0; t < ntl && !failed; t++) {
             int Er[ITEMS], Ei[ITEMS];
             bool out[ITEMS] = {};  // the group is outside the fixed-point range, or its sums would lose too much
-            if (a.diag) {      // amplitudes with a diagonal entry of their own: scaled to what else is in their column, or 0
+            if (SPEC && a.diag) {  // amplitudes with a diagonal entry of their own: scaled to what else is in their column, or 0
                 const unsigned long long mine = a.diag >> kc;
 #pragma unroll
                 for (int it = 0; it < ITEMS; it++)
@@ -324,7 +326,7 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
                         if (!mag_bits(x[it][e].y)) low |= (unsigned)__double2loint(x[it][e].y);
                     }
                 out[it] |= Er[it] < kMinExp || Er[it] > kMaxExp || Ei[it] < kMinExp || Ei[it] > kMaxExp || low;
-                if (a.check) {  // by the larger part of an amplitude
+                if (SPEC && a.check) {  // by the larger part of an amplitude
                     const int E = PARTS ? max(mr ? Er[it] : 0, mi ? Ei[it] : 0) : Er[it];
                     const bool zero = mr == 0 && mi == 0;
                     if (!__all_sync(~0u, (int)(ml >> 20) >= E - a.reach || zero)) {
@@ -490,7 +492,7 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
                     }
                     __syncwarp();
                     // a function of its own: with the FP64 products as a condition here the FP64 pipe was 69 % busy
-                    if (a.diag || skip) store_spec<MODE>(a, st, base + off, h, s, lane, skip);
+                    if ((SPEC && a.diag) || skip) store_spec<MODE>(a, st, base + off, h, s, lane, skip);
                     else store_body<MODE, false>(a, st, base + off, h, s, lane, 0u);
                 }
             }
@@ -615,18 +617,18 @@ static int mode_of(const Op &op) {
     return k == 5 ? C5 : k == 4 ? C4 : -1;
 }
 
-template <int MODE>
+template <int MODE, bool SPEC>
 static void launch(const Args &a, int sms, cudaStream_t st) {
     using C = Cfg<MODE>;
     static bool attr = false;
     if (!attr) {
         const cudaError_t e =
-            cudaFuncSetAttribute(dense_f64_tc_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+            cudaFuncSetAttribute(dense_f64_tc_kernel<MODE, SPEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
         if (e != cudaSuccess) throw Error(QSIM_ECUDA, std::string("dense_f64_tc_kernel attribute: ") + cudaGetErrorString(e));
         attr = true;
     }
     // one CTA per SM: it holds all 512 tensor-memory columns
-    dense_f64_tc_kernel<MODE><<<(int)std::min<long long>(a.ntiles, sms), kThreads, C::SMEM, st>>>(a);
+    dense_f64_tc_kernel<MODE, SPEC><<<(int)std::min<long long>(a.ntiles, sms), kThreads, C::SMEM, st>>>(a);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) throw Error(QSIM_ECUDA, std::string("dense_f64_tc_kernel: ") + cudaGetErrorString(e));
     note_launches(1, QSIM_KERNEL_DENSE_TC);
@@ -701,7 +703,7 @@ bool launch_dense_f64_tc(void *state, int n, const Op &op, const void *dig, cons
     std::sort(fix.begin(), fix.end());
     a.nfix = (int)fix.size();
     for (int i = 0; i < a.nfix; i++) a.fix[i] = fix[i];
-#define QSIM_LAUNCH(M) launch<M>(a, sms, st)
+#define QSIM_LAUNCH(M) (a.diag || a.check) ? launch<M, true>(a, sms, st) : launch<M, false>(a, sms, st)
     QSIM_F64TC_SWITCH(mode, QSIM_LAUNCH)
 #undef QSIM_LAUNCH
     return true;
