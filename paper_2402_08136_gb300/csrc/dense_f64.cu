@@ -31,7 +31,8 @@
 // controlled gate written as a dense one, the diagonal of a gate close to the identity) are multiplied in FP64 on the way
 // out, and neither they nor their amplitudes count in the scales of the rest.
 // A tile with a group that is not finite, whose largest exponent is far from 1, or whose sums would lose more than FP64
-// ones is computed in the plain FP64 form by the same warp (plain_tile).
+// ones is computed in the plain FP64 form by the same warp (plain_tile; from 4 targets on and where the groups are tested,
+// that group alone: plain_groups).
 //
 // 26 qubits, FP64 form -> this one, TB/s: k = 1 2.26 -> 3.83, 2 1.17 -> 3.8, 3 0.62 -> 3.8, 4 0.31 -> 2.45, 5 0.16 -> 1.35,
 // 6 0.072 -> 0.76 (from 4 targets on, large states take dense_f64_tc.cu).  k <= 3 is bound by issue slots (splitting and
@@ -132,6 +133,51 @@ __device__ __noinline__ void plain_tile(const Args &a, char *base, int lane) {
 #pragma unroll 1
     for (int o = 0; o < OUT; o++) {
         *reinterpret_cast<double2 *>(p + a.amp[lane % LPG + o * LPG]) = y[o];
+    }
+    __syncwarp();
+}
+
+// The groups of a tile in mask gm in FP64 (K >= 4), a warp per group (two with 4 targets): a lane loads its amplitudes and
+// has their rows, U's columns come in order, the column's amplitude from its lane.
+template <int K, bool REALU>
+__device__ __noinline__ void plain_groups(const Args &a, char *base, unsigned gm, int lane) {
+    constexpr int D = 1 << K, L = D < 32 ? D : 32, ROWS = D / L;  // lanes per group, rows per lane
+    const int r = lane % L;
+    while (gm) {
+        int g = __ffs(gm) - 1;
+        bool mine = true;
+        gm &= gm - 1;
+        if (L < 32 && lane >= L) {
+            mine = gm != 0;
+            if (mine) g = __ffs(gm) - 1;
+        }
+        if (L < 32) gm &= gm - 1;
+        char *p = base + a.col[g];
+        double2 x[ROWS], y[ROWS];
+#pragma unroll
+        for (int o = 0; o < ROWS; o++) {
+            x[o] = *reinterpret_cast<const double2 *>(p + a.amp[r + 32 * o]);
+            y[o] = make_double2(0.0, 0.0);
+        }
+#pragma unroll
+        for (int h = 0; h < ROWS; h++)
+#pragma unroll 4
+            for (int c = 0; c < L; c++) {
+                const double zx = __shfl_sync(~0u, x[h].x, c, L), zy = __shfl_sync(~0u, x[h].y, c, L);
+#pragma unroll
+                for (int o = 0; o < ROWS; o++) {
+                    const double2 *w = a.Ut + (c + 32 * h) * D + r + 32 * o;
+                    const double2 u = REALU ? make_double2(__ldg(&w->x), 0.0) : __ldg(w);
+                    y[o].x = fma(u.x, zx, y[o].x);
+                    if (!REALU) y[o].x = fma(-u.y, zy, y[o].x);
+                    y[o].y = fma(u.x, zy, y[o].y);
+                    if (!REALU) y[o].y = fma(u.y, zx, y[o].y);
+                }
+            }
+        __syncwarp();  // every output of a group is computed before any is stored
+        if (mine)
+#pragma unroll
+            for (int o = 0; o < ROWS; o++) *reinterpret_cast<double2 *>(p + a.amp[r + 32 * o]) = y[o];
     }
     __syncwarp();
 }
@@ -308,9 +354,16 @@ __global__ void __launch_bounds__(Cfg<K, REALU>::THREADS, 1) dense_f64_kernel(co
                     }
             }
             if (C::PREFETCH && i == NT - 1 && t + warps < a.ntasks) load(t + warps, x);
+            unsigned gm = 0;  // groups in FP64
             if (!__all_sync(~0u, fits)) {
-                plain_tile<K, REALU>(a, tb, lane);
-                continue;
+                if constexpr (SPEC && !C::RF) {
+                    gm = __reduce_or_sync(~0u, fits ? 0u : 1u << (REALU ? n >> 1 : (n & 1) * 4 + (n >> 1)));
+                    plain_groups<K, REALU>(a, tb, gm, lane);
+                    if (gm == (1u << (1 << C::GB)) - 1u) continue;
+                } else {
+                    plain_tile<K, REALU>(a, tb, lane);
+                    continue;
+                }
             }
             // result exponents of this lane's two accumulator columns 2 q, 2 q + 1 (and row n)
             const int ep = E0 | (E1 << 16);
@@ -361,7 +414,7 @@ __global__ void __launch_bounds__(Cfg<K, REALU>::THREADS, 1) dense_f64_kernel(co
                         for (int h = 0; h < 2; h++) {  // amplitudes n and n + 8 of group q
                             const int row = 16 * mt + 8 * h + n;
                             const double2 y = make_double2(join<C::BIAS>(acc[2 * h], a.sh, ex[0]), join<C::BIAS>(acc[2 * h + 1], a.sh, ex[1]));
-                            put<K, SPEC>(a, row, ob + a.amp[16 * mt + 8 * h], y);
+                            if (!SPEC || !((gm >> q) & 1u)) put<K, SPEC>(a, row, ob + a.amp[16 * mt + 8 * h], y);
                         }
                     } else {
                         double re[4];
@@ -383,7 +436,8 @@ __global__ void __launch_bounds__(Cfg<K, REALU>::THREADS, 1) dense_f64_kernel(co
                         for (int c = 0; c < 4; c++) {  // amplitudes n and n + 8 of groups q and q + 4
                             const int row = 16 * mt + 8 * (c >> 1) + n;
                             const double2 y = make_double2(re[c], join<C::BIAS>(acc[c], a.sh, ex[c & 1]));
-                            put<K, SPEC>(a, row, ob + a.col[4 * (c & 1)] + a.amp[16 * mt + 8 * (c >> 1)], y);
+                            if (!SPEC || !((gm >> (q + 4 * (c & 1))) & 1u))
+                                put<K, SPEC>(a, row, ob + a.col[4 * (c & 1)] + a.amp[16 * mt + 8 * (c >> 1)], y);
                         }
                     }
                 }
@@ -667,7 +721,7 @@ void dense_f64_pack_scales(const Op &op, unsigned char *out) {
 //     bytes that is never above S (f64_digits.cuh, rows_fit).  A row with an entry multiplied in FP64 is safe too
 //     while that product alone bounds the error of the rest: from an exponent of its amplitude on (`from`).
 // A group has an amplitude of 128 units at least, so a U without small entries is safe for every state (most Haar
-// gates of up to 3 targets).  With others every group is tested, and one that fails runs in FP64 (in dense_f64.cu its
+// gates of up to 3 targets).  With others every group is tested, and one that fails runs in FP64 (up to 3 targets its
 // tile).  The four lanes that hold a group look at their own largest amplitudes first: with one of 2^(7 - reach) units
 // in each, whichever columns they are in, a row has at least its smallest entry of every lane's columns times that.  A
 // gate with rows that fail even where all amplitudes are within a factor of two of each other stays in FP64 as a whole.
