@@ -36,8 +36,8 @@
 //
 // 26 qubits, FP64 form -> this one, TB/s: k = 1 2.26 -> 3.83, 2 1.17 -> 3.8, 3 0.62 -> 3.8, 4 0.31 -> 2.45, 5 0.16 -> 1.35,
 // 6 0.072 -> 0.76 (from 4 targets on, large states take dense_f64_tc.cu).  k <= 3 is bound by issue slots (splitting and
-// joining the digits), wider gates by the MMAs.  Gates with small entries, whose groups are tested, 25 qubits: real 2 and
-// 4 targets 295 -> 391 and 291 -> 371 us (Haar), 1 target close to the identity 288 -> 397 us (FP64 485 us).  Error against long
+// joining the digits), wider gates by the MMAs.  Gates with small entries, whose groups are tested, 25 qubits: real 2, 4
+// and 5 targets 295 -> 340, 291 -> 379, 432 -> 488 us (Haar), 1 target close to the identity 288 -> 346 us (FP64 485 us).  Error against long
 // double 4.6e-17 of the largest amplitude (FP64 form 7e-17 to 3.5e-16).
 #include <cuda_runtime.h>
 #include <cuda_fp16.h>
