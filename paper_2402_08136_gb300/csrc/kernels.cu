@@ -1656,7 +1656,8 @@ void mark_replays(const hhl_circuit *h, qsim_circuit *c, void *stream) {
     std::lock_guard<std::mutex> lk(mark->mu);
     cudaEvent_t &ev = mark->event[dev];
     if (ev == nullptr) CUDA_OK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
-    CUDA_OK(cudaEventRecordWithFlags(ev, st, cudaEventRecordExternal));
+    // where a graph may not hold such a node, the order is the caller's
+    if (cudaEventRecordWithFlags(ev, st, cudaEventRecordExternal) != cudaSuccess) cudaGetLastError();
 }
 
 void after_replays(const hhl_circuit *h, void *stream) {
