@@ -213,10 +213,11 @@ __global__ void __launch_bounds__(Cfg<K, REALU>::THREADS, 1) dense_f64_kernel(co
     constexpr int NT = C::NT, EPL = C::EPL, KS = C::KS;
     extern __shared__ __align__(16) uint4 tabs[];  // [TABS][MT][KS][digit][lane]
     const int tid = threadIdx.x, lane = tid & 31, q = lane & 3, n = lane >> 2;
-    for (int i = tid; i < C::TAB * (C::TABS == 3 ? 2 : 1); i += blockDim.x) {
+    constexpr int IN = C::TAB * (C::TABS == 3 ? 2 : 1);  // tables in memory, the rows' bytes behind them
+    for (int i = tid; i < IN + (SPEC && a.check ? C::ROWS / 16 : 0); i += blockDim.x) {
         uint4 v = a.dig[i];
-        tabs[i] = v;
-        if (C::TABS == 3 && i >= C::TAB) {  // -Im U
+        tabs[i < IN ? i : i - IN + C::TABS * C::TAB] = v;
+        if (C::TABS == 3 && i >= C::TAB && i < IN) {  // -Im U
             v.x ^= 0x80008000u;
             v.y ^= 0x80008000u;
             v.z ^= 0x80008000u;
@@ -225,9 +226,6 @@ __global__ void __launch_bounds__(Cfg<K, REALU>::THREADS, 1) dense_f64_kernel(co
         }
     }
     const unsigned char *rows = reinterpret_cast<const unsigned char *>(tabs + C::TABS * C::TAB);
-    if (SPEC && a.check)
-        for (int i = tid; i < C::ROWS / 16; i += blockDim.x)
-            tabs[C::TABS * C::TAB + i] = a.dig[C::TAB * (C::TABS == 3 ? 2 : 1) + i];
     __syncthreads();
     const int wpc = blockDim.x / 32;
     const long long warps = (long long)gridDim.x * wpc;

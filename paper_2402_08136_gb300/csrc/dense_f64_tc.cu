@@ -228,9 +228,8 @@ __global__ void __launch_bounds__(kThreads, 1) dense_f64_tc_kernel(const __grid_
     unsigned *tslot = reinterpret_cast<unsigned *>(drain + 1);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    for (int i = tid; i < C::BBYTES / 16; i += kThreads) reinterpret_cast<uint4 *>(sm)[i] = a.dig[i];
-    if (SPEC && a.check)
-        for (int i = tid; i < C::ROWS / 16; i += kThreads) reinterpret_cast<uint4 *>(rows)[i] = a.dig[C::BBYTES / 16 + i];
+    for (int i = tid; i < C::BBYTES / 16 + (SPEC && a.check ? C::ROWS / 16 : 0); i += kThreads)
+        reinterpret_cast<uint4 *>(i < C::BBYTES / 16 ? sm : rows - C::BBYTES)[i] = a.dig[i];
     if (tid == 0) {
         for (int i = 0; i < SLOTS; i++) {
             mbar_init(&full[i], kProdWarps);
